@@ -8,11 +8,13 @@
 
 namespace wsn {
 
-// C = op(A) op(B) with A(m, k) = A[m sam + k sak] and B(k, n) = B[k sbk + n sbn] (BF16),
-// M x N x K; the epilogue decides what is written (see Epi).
+// C = op(A) op(B), M x N x K in BF16; the epilogue decides what is written (see Epi).  Each
+// operand is stored with one of its dimensions contiguous (the kernel's AK / BK: that is K)
+// and ld elements between neighbours of the other.
 struct Gemm {
     const __nv_bfloat16 *A, *B;
-    long long sam, sak, sbk, sbn;
+    int lda, ldb;
+    int avec, bvec;           // 16-byte copies: the pointer is 16-byte aligned, ld a multiple of 8
     int M, N, K;
     const float *bias;        // per column (BIAS, BIAS_GELU)
     const float *scale;       // per column, BIAS only: out = (C + bias) * scale (NULL: 1)
@@ -39,85 +41,216 @@ __device__ __forceinline__ void mma_bf16(float *c, const unsigned *a, const unsi
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-constexpr int TM = 64, TN = 64, TK = 32, PAD = 8;
+constexpr int TM = 64, TN = 64, TK = 32, STAGES = 3;
+// one operand's tile in shared memory: 64 rows of 32 K values (rows padded to 40) or 32 K rows
+// of 64 values (padded to 72); both pads put the eight 16-byte rows that an ldmatrix reads at
+// once into different banks
+constexpr int LDK = TK + 8, LDMN = TM + 8;
+constexpr int TILE = TM * LDK > TK * LDMN ? TM * LDK : TK * LDMN;
 
-// 4 warps in a 2 x 2 arrangement, each computing a 32 x 32 block of C as 2 x 4 tiles of
-// m16n8.  Shared tiles: As[m][k] and Bs[n][k], k contiguous, rows padded by 8 BF16 so the
-// 32-bit fragment loads of a warp hit 32 distinct banks.
-template <int EPI>
-__global__ void __launch_bounds__(128) gemm_kernel(Gemm g)
+__device__ __forceinline__ unsigned sm_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void ldsm4(unsigned *r, unsigned addr)
 {
-    __shared__ __align__(16) __nv_bfloat16 As[TM][TK + PAD];
-    __shared__ __align__(16) __nv_bfloat16 Bs[TN][TK + PAD];
-    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+
+__device__ __forceinline__ void ldsm4t(unsigned *r, unsigned addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+
+// Rows x0 .. x0 + 63 of the non-K dimension (limit X) by k0 .. k0 + 31 (limit kend) into one
+// stage, zeros outside: 16-byte asynchronous copies along the contiguous dimension, or (no
+// such alignment: a width of 7) element by element, neighbouring threads on neighbouring
+// addresses.
+template <bool KC>
+__device__ __forceinline__ void load_tile(__nv_bfloat16 *dst, const __nv_bfloat16 *src, int ld, bool vec,
+                                          int x0, int X, int k0, int kend)
+{
+    constexpr int INNER = KC ? TK : TM, OUTER = KC ? TM : TK, LDS = KC ? LDK : LDMN;
+    const int i0 = KC ? k0 : x0, ilim = KC ? kend : X, o0 = KC ? x0 : k0, olim = KC ? X : kend;
+    if (vec) {
+        // (the contiguous dimension spans whole rows of ld = a multiple of 8: a chunk is in or out)
+        for (int c = threadIdx.x; c < OUTER * (INNER / 8); c += 128) {
+            const int o = c / (INNER / 8), i = (c % (INNER / 8)) * 8;
+            const bool in = o0 + o < olim && i0 + i < ilim;
+            const __nv_bfloat16 *p = in ? src + (long long)(o0 + o) * ld + i0 + i : src;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                         ::"r"(sm_addr(dst + o * LDS + i)), "l"(p), "r"(in ? 16 : 0) : "memory");
+        }
+    } else {
+        for (int c = threadIdx.x; c < OUTER * INNER; c += 128) {
+            const int o = c / INNER, i = c % INNER;
+            const bool in = o0 + o < olim && i0 + i < ilim;
+            dst[o * LDS + i] = in ? src[(long long)(o0 + o) * ld + i0 + i] : __float2bfloat16(0.0f);
+        }
+    }
+}
+
+// The K range [kb, ke) of one 64 x 64 tile of C (128 threads): 4 warps in a 2 x 2
+// arrangement, each a 32 x 32 block as 2 x 4 tiles of m16n8, K ascending in steps of 16 (the
+// order of the sums does not depend on the tile's operand layout).  Three stages of 32 K
+// values in flight.  COLSUM: with csum given, threads 0 .. 63 also sum the columns of B
+// in K order.
+// These layers are latency-bound, not tensor-bound (a 4096-row layer is 0.5 GFLOP), so the
+// pipeline depth and the coalesced copies matter, not the instruction.
+template <bool AK, bool BK, bool COLSUM>
+__device__ __forceinline__ void gemm_tile(const Gemm &g, int m0, int n0, int kb, int ke,
+                                          float (*acc)[4][4], float *csum)
+{
+    __shared__ __align__(16) __nv_bfloat16 As[STAGES][TILE], Bs[STAGES][TILE];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-    const int gq = lane >> 2, tq = lane & 3;
-    float acc[2][4][4];
+    const int steps = (ke - kb + TK - 1) / TK;
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.0f;
-    const __nv_bfloat16 zero = __float2bfloat16(0.0f);
-    for (int k0 = 0; k0 < g.K; k0 += TK) {
-        for (int e = threadIdx.x; e < TM * TK; e += 128) {
-            const int r = e / TK, c = e - r * TK;
-            const int m = m0 + r, n = n0 + r, k = k0 + c;
-            As[r][c] = (m < g.M && k < g.K) ? g.A[m * g.sam + k * g.sak] : zero;
-            Bs[r][c] = (n < g.N && k < g.K) ? g.B[k * g.sbk + n * g.sbn] : zero;
+    auto fill = [&](int t) {
+        if (t < steps) {
+            load_tile<AK>(As[t % STAGES], g.A, g.lda, g.avec, m0, g.M, kb + t * TK, ke);
+            load_tile<BK>(Bs[t % STAGES], g.B, g.ldb, g.bvec, n0, g.N, kb + t * TK, ke);
         }
-        __syncthreads();
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int t = 0; t < STAGES - 1; ++t) fill(t);
+    // ldmatrix source of a lane: matrix lane / 8, row lane % 8
+    const int q8 = lane >> 3, r8 = lane & 7;
+    for (int t = 0; t < steps; ++t) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+        __syncthreads();                      // stage t landed; stage t - 1 is free again
+        fill(t + STAGES - 1);
+        const __nv_bfloat16 *as = As[t % STAGES], *bs = Bs[t % STAGES];
 #pragma unroll
         for (int kk = 0; kk < TK; kk += 16) {
-            unsigned a[2][4], b[4][2];
+            unsigned a[2][4], b[2][4];
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
-                const int row = wm + 16 * i + gq;
-                a[i][0] = *reinterpret_cast<const unsigned *>(&As[row][kk + 2 * tq]);
-                a[i][1] = *reinterpret_cast<const unsigned *>(&As[row + 8][kk + 2 * tq]);
-                a[i][2] = *reinterpret_cast<const unsigned *>(&As[row][kk + 2 * tq + 8]);
-                a[i][3] = *reinterpret_cast<const unsigned *>(&As[row + 8][kk + 2 * tq + 8]);
+                // matrices (m, k), (m + 8, k), (m, k + 8), (m + 8, k + 8)
+                const int m = wm + 16 * i;
+                if (AK) ldsm4(a[i], sm_addr(as + (m + (q8 & 1) * 8 + r8) * LDK + kk + (q8 >> 1) * 8));
+                else ldsm4t(a[i], sm_addr(as + (kk + (q8 >> 1) * 8 + r8) * LDMN + m + (q8 & 1) * 8));
             }
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int col = wn + 8 * j + gq;
-                b[j][0] = *reinterpret_cast<const unsigned *>(&Bs[col][kk + 2 * tq]);
-                b[j][1] = *reinterpret_cast<const unsigned *>(&Bs[col][kk + 2 * tq + 8]);
+            for (int j = 0; j < 2; ++j) {
+                // matrices (n, k), (n, k + 8), (n + 8, k), (n + 8, k + 8)
+                const int n = wn + 16 * j;
+                if (BK) ldsm4(b[j], sm_addr(bs + (n + (q8 >> 1) * 8 + r8) * LDK + kk + (q8 & 1) * 8));
+                else ldsm4t(b[j], sm_addr(bs + (kk + (q8 & 1) * 8 + r8) * LDMN + n + (q8 >> 1) * 8));
             }
 #pragma unroll
             for (int i = 0; i < 2; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], a[i], b[j]);
+                for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], a[i], &b[j >> 1][2 * (j & 1)]);
         }
-        __syncthreads();
+        if (COLSUM && csum && threadIdx.x < TN) {
+            float s = *csum;
+            for (int k = 0; k < TK; ++k) s += __bfloat162float(bs[k * LDMN + threadIdx.x]);
+            *csum = s;
+        }
     }
-    // accumulator (i, j, q): row wm + 16 i + gq (+ 8 for q >= 2), column wn + 8 j + 2 tq + (q & 1)
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// accumulator (i, j, q) of a thread: row wm + 16 i + gq (+ 8 for q >= 2), column
+// wn + 8 j + 2 tq + (q & 1)
+template <int EPI>
+__device__ __forceinline__ void gemm_store(const Gemm &g, int m0, int n0, float (*acc)[4][4])
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32, gq = lane >> 2, tq = lane & 3;
+    // neighbouring columns in one store: even N (n is even) and an 8-byte aligned output
+    const bool pair = !(g.N & 1) && !((size_t)(EPI == EPI_GELU_BWD ? (const void *)g.act : (const void *)g.out) & 7);
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int m = m0 + wm + 16 * i + gq + (q >= 2 ? 8 : 0);
-                const int n = n0 + wn + 8 * j + 2 * tq + (q & 1);
+            for (int h = 0; h < 2; ++h) {
+                const int m = m0 + wm + 16 * i + gq + 8 * h, n = n0 + wn + 8 * j + 2 * tq;
                 if (m >= g.M || n >= g.N) continue;
                 const long long o = (long long)m * g.N + n;
-                const float c = acc[i][j][q];
-                if (EPI == EPI_STORE) {
-                    g.out[o] = c;
-                } else if (EPI == EPI_BIAS) {
-                    g.out[o] = g.scale ? (c + g.bias[n]) * g.scale[n] : c + g.bias[n];
-                } else if (EPI == EPI_BIAS_GELU) {
-                    const float u = c + g.bias[n];
-                    g.out[o] = u;
-                    g.act[o] = __float2bfloat16(gelu_f(u));
-                } else {
-                    g.act[o] = __float2bfloat16(c * gelu_grad_f(g.pre[o]));
+                const bool two = n + 1 < g.N;
+                float c[2], u[2];
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    c[q] = acc[i][j][2 * h + q];
+                    if (q && !two) continue;
+                    if (EPI == EPI_BIAS) c[q] = g.scale ? (c[q] + g.bias[n + q]) * g.scale[n + q] : c[q] + g.bias[n + q];
+                    if (EPI == EPI_BIAS_GELU) { c[q] = c[q] + g.bias[n + q]; u[q] = gelu_f(c[q]); }
+                    if (EPI == EPI_GELU_BWD) u[q] = c[q] * gelu_grad_f(g.pre[o + q]);
+                }
+                if (EPI != EPI_GELU_BWD) {
+                    if (pair) *reinterpret_cast<float2 *>(g.out + o) = make_float2(c[0], c[1]);
+                    else { g.out[o] = c[0]; if (two) g.out[o + 1] = c[1]; }
+                }
+                if (EPI == EPI_BIAS_GELU || EPI == EPI_GELU_BWD) {
+                    if (pair) *reinterpret_cast<__nv_bfloat162 *>(g.act + o) = __floats2bfloat162_rn(u[0], u[1]);
+                    else { g.act[o] = __float2bfloat16(u[0]); if (two) g.act[o + 1] = __float2bfloat16(u[1]); }
                 }
             }
         }
+    }
+}
+
+// A layer: A with K contiguous (activations or output gradients, a row per sample), B the
+// weights (N contiguous forward, K contiguous backward).
+template <int EPI, bool BK>
+__global__ void __launch_bounds__(128) gemm_kernel(Gemm g)
+{
+    float acc[2][4][4];
+    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+    gemm_tile<true, BK, false>(g, m0, n0, 0, g.K, acc, nullptr);
+    gemm_store<EPI>(g, m0, n0, acc);
+}
+
+// Weight and bias gradients of up to kGroup layers in one launch: dW = act^T g and the column
+// sums of g.  K is the batch, so a layer has few tiles and long sums (256 x 256 weights: 16
+// tiles of 4096 terms each); the batch is split over blockIdx.y (chunks of `chunk` rows), each
+// split writes its own partial gradient and grad_reduce_kernel adds the splits in order
+// (deterministic).  With one launch per layer, unsplit, element-wise strided loads and a
+// separate column-sum kernel of 8 blocks, the gradients of a 4096-row minibatch took 1520 us; with
+// this 131 us (11 launches, none of them above a few microseconds of work).
+constexpr int kGroup = 8;
+struct WgradGroup {
+    Gemm g[kGroup];
+    long long woff[kGroup], boff[kGroup];
+    int tile0[kGroup + 1];    // first tile of each layer
+    int layers, chunk;
+    long long stride;         // floats between the splits' partial gradients
+    float *part;
+};
+
+__global__ void __launch_bounds__(128) wgrad_kernel(const __grid_constant__ WgradGroup w)
+{
+    int l = 0;
+    while (l + 1 < w.layers && (int)blockIdx.x >= w.tile0[l + 1]) ++l;
+    Gemm g = w.g[l];
+    const int tile = blockIdx.x - w.tile0[l], nt = (g.N + TN - 1) / TN;
+    const int m0 = tile / nt * TM, n0 = tile % nt * TN;
+    const int kb = blockIdx.y * w.chunk, ke = min(g.K, kb + w.chunk);
+    float *part = w.part + blockIdx.y * w.stride;
+    g.out = part + w.woff[l];
+    float acc[2][4][4], csum = 0.0f;
+    gemm_tile<false, false, true>(g, m0, n0, kb, ke, acc, m0 == 0 ? &csum : nullptr);
+    gemm_store<EPI_STORE>(g, m0, n0, acc);
+    if (m0 == 0 && threadIdx.x < TN && n0 + (int)threadIdx.x < g.N)
+        part[w.boff[l] + n0 + threadIdx.x] = csum;
+}
+
+__global__ void grad_reduce_kernel(const float *part, long long stride, int splits, float *grad,
+                                   long long n)
+{
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x) {
+        float s = part[i];
+        for (int k = 1; k < splits; ++k) s += part[k * stride + i];
+        grad[i] = s;
     }
 }
 
@@ -186,27 +319,6 @@ __global__ void column_stats_kernel(const float *x, long long ld, int B, int D, 
             const double rms = sqrt(ms);
             second[d] = rms > 0.0 ? (float)rms : 1.0f;
         }
-    }
-}
-
-// column sums of a B x N BF16 matrix into FP32 (bias gradients).  A block of 32 x 8 threads
-// takes 32 columns: each of its 8 row groups sums rows g, g + 8, ... in order, then the 8
-// partial sums are added in group order (a fixed order: deterministic).
-__global__ void __launch_bounds__(256) column_sum_kernel(const __nv_bfloat16 *g, int B, int N, float *out)
-{
-    __shared__ float part[8][33];
-    const int c = threadIdx.x & 31, r = threadIdx.x >> 5;
-    const int n = blockIdx.x * 32 + c;
-    float s = 0.0f;
-    if (n < N)
-        for (int b = r; b < B; b += 8) s += __bfloat162float(g[(long long)b * N + n]);
-    part[r][c] = s;
-    __syncthreads();
-    if (r == 0 && n < N) {
-        float t = 0.0f;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) t += part[q][c];
-        out[n] = t;
     }
 }
 

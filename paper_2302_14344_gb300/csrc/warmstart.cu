@@ -32,7 +32,9 @@ struct wsn_s {
     std::vector<__nv_bfloat16 *> act;  // act[l]: input of layer l (B x sizes[l])
     std::vector<float *> pre;          // pre[l]: pre-activation of hidden layer l (B x sizes[l+1])
     float *y = nullptr;                // network output (B x out)
-    __nv_bfloat16 *g0 = nullptr, *g1 = nullptr;   // layer gradients (B x max width)
+    std::vector<__nv_bfloat16 *> gl;   // gl[l]: gradient of layer l's output (B x sizes[l+1])
+    float *part = nullptr;             // partial weight gradients of the batch's splits
+    int max_splits = 1;
     // fused tensor-core inference (the 32-256-256-256-7 warm-start shape): packed BF16
     // weights (K-major per layer), their tensor maps, the kernel's error word
     __nv_bfloat16 *wpack[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -67,8 +69,10 @@ void free_ws(wsn_t w)
     for (auto *q : w->pre) cudaFree(q);
     w->act.clear();
     w->pre.clear();
-    cudaFree(w->y); cudaFree(w->g0); cudaFree(w->g1);
-    w->y = nullptr; w->g0 = nullptr; w->g1 = nullptr;
+    for (auto *q : w->gl) cudaFree(q);
+    w->gl.clear();
+    cudaFree(w->y); cudaFree(w->part);
+    w->y = nullptr; w->part = nullptr;
     w->cap = 0;
 }
 
@@ -78,27 +82,41 @@ int reserve(wsn_t w, int batch)
     free_ws(w);
     const int L = (int)w->sizes.size() - 1;
     const int cap = std::max(batch, 1024);
-    int wmax = 0;
-    for (int s : w->sizes) wmax = std::max(wmax, s);
     w->act.assign(L, nullptr);
     w->pre.assign(L, nullptr);
+    w->gl.assign(L, nullptr);
+    // splits of the batch in the weight gradients: enough 64 x 64 tiles for two blocks per SM
+    // and scheduling slot (about 600), at most 16 (each holds a whole partial gradient)
+    long long tiles = 0;
+    for (int l = 0; l < L; ++l)
+        tiles += (long long)((w->sizes[l] + wsn::TM - 1) / wsn::TM) * ((w->sizes[l + 1] + wsn::TN - 1) / wsn::TN);
+    w->max_splits = (int)std::max<long long>(1, std::min<long long>(16, (600 + tiles - 1) / tiles));
+    WCK(cudaMalloc((void **)&w->part, sizeof(float) * (size_t)w->nparams * w->max_splits), "cudaMalloc");
     for (int l = 0; l < L; ++l) {
         WCK(cudaMalloc((void **)&w->act[l], sizeof(__nv_bfloat16) * (size_t)cap * w->sizes[l]), "cudaMalloc");
         WCK(cudaMalloc((void **)&w->pre[l], sizeof(float) * (size_t)cap * w->sizes[l + 1]), "cudaMalloc");
+        WCK(cudaMalloc((void **)&w->gl[l], sizeof(__nv_bfloat16) * (size_t)cap * w->sizes[l + 1]), "cudaMalloc");
     }
     WCK(cudaMalloc((void **)&w->y, sizeof(float) * (size_t)cap * w->sizes[L]), "cudaMalloc");
-    WCK(cudaMalloc((void **)&w->g0, sizeof(__nv_bfloat16) * (size_t)cap * wmax), "cudaMalloc");
-    WCK(cudaMalloc((void **)&w->g1, sizeof(__nv_bfloat16) * (size_t)cap * wmax), "cudaMalloc");
     w->cap = cap;
     w->ws_gen = ++g_ws_generation;
     return SIM_OK;
 }
 
-template <int EPI>
+// operands of a product, and whether their rows can be copied 16 bytes at a time
+wsn::Gemm operands(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int ldb)
+{
+    wsn::Gemm g{};
+    g.A = A; g.lda = lda; g.avec = lda % 8 == 0 && ((uintptr_t)A & 15) == 0;
+    g.B = B; g.ldb = ldb; g.bvec = ldb % 8 == 0 && ((uintptr_t)B & 15) == 0;
+    return g;
+}
+
+template <int EPI, bool BK>
 int gemm(wsn_t w, const wsn::Gemm &g, cudaStream_t st)
 {
     dim3 grid((g.N + wsn::TN - 1) / wsn::TN, (g.M + wsn::TM - 1) / wsn::TM);
-    wsn::gemm_kernel<EPI><<<grid, 128, 0, st>>>(g);
+    wsn::gemm_kernel<EPI, BK><<<grid, 128, 0, st>>>(g);
     WCK(cudaGetLastError(), "gemm launch");
     return SIM_OK;
 }
@@ -114,19 +132,17 @@ int forward(wsn_t w, const float *x, long long ldx, int batch, bool scaled, cuda
         x, ldx, w->mean, w->inv_std, w->act[0], batch, w->sizes[0]);
     WCK(cudaGetLastError(), "normalize launch");
     for (int l = 0; l < L; ++l) {
-        wsn::Gemm g{};
-        g.A = w->act[l]; g.sam = w->sizes[l]; g.sak = 1;
-        g.B = w->pb + w->w_off[l]; g.sbk = w->sizes[l + 1]; g.sbn = 1;
+        wsn::Gemm g = operands(w->act[l], w->sizes[l], w->pb + w->w_off[l], w->sizes[l + 1]);
         g.M = batch; g.N = w->sizes[l + 1]; g.K = w->sizes[l];
         g.bias = w->p + w->b_off[l];
         if (l < L - 1) {
             g.out = w->pre[l];
             g.act = w->act[l + 1];
-            if ((rc = gemm<wsn::EPI_BIAS_GELU>(w, g, st))) return rc;
+            if ((rc = gemm<wsn::EPI_BIAS_GELU, false>(w, g, st))) return rc;
         } else {
             g.out = w->y;
             g.scale = scaled ? w->scale : nullptr;
-            if ((rc = gemm<wsn::EPI_BIAS>(w, g, st))) return rc;
+            if ((rc = gemm<wsn::EPI_BIAS, false>(w, g, st))) return rc;
         }
     }
     return SIM_OK;
@@ -139,30 +155,42 @@ int backward(wsn_t w, const float *t, const float *mask, int batch, float *grad,
     const int L = (int)w->sizes.size() - 1;
     const int N = w->sizes[L];
     wsn::output_grad_kernel<<<grid_for((long long)batch * N), 256, 0, st>>>(
-        w->y, t, mask, w->scale, w->g0, batch, N, loss);
+        w->y, t, mask, w->scale, w->gl[L - 1], batch, N, loss);
     WCK(cudaGetLastError(), "output grad launch");
-    __nv_bfloat16 *gcur = w->g0, *gnext = w->g1;
     int rc;
-    for (int l = L - 1; l >= 0; --l) {
+    for (int l = L - 1; l > 0; --l) {           // g_prev = (g W^T) * GELU'(pre)
         const int in = w->sizes[l], out = w->sizes[l + 1];
-        wsn::Gemm gw{};                         // dW = act^T g
-        gw.A = w->act[l]; gw.sam = 1; gw.sak = in;
-        gw.B = gcur; gw.sbk = out; gw.sbn = 1;
-        gw.M = in; gw.N = out; gw.K = batch;
-        gw.out = grad + w->w_off[l];
-        if ((rc = gemm<wsn::EPI_STORE>(w, gw, st))) return rc;
-        wsn::column_sum_kernel<<<(out + 31) / 32, 256, 0, st>>>(gcur, batch, out, grad + w->b_off[l]);
-        WCK(cudaGetLastError(), "column sum launch");
-        if (l > 0) {                            // g_prev = (g W^T) * GELU'(pre)
-            wsn::Gemm ga{};
-            ga.A = gcur; ga.sam = out; ga.sak = 1;
-            ga.B = w->pb + w->w_off[l]; ga.sbk = 1; ga.sbn = out;
-            ga.M = batch; ga.N = in; ga.K = out;
-            ga.pre = w->pre[l - 1];
-            ga.act = gnext;
-            if ((rc = gemm<wsn::EPI_GELU_BWD>(w, ga, st))) return rc;
-            std::swap(gcur, gnext);
+        wsn::Gemm ga = operands(w->gl[l], out, w->pb + w->w_off[l], out);
+        ga.M = batch; ga.N = in; ga.K = out;
+        ga.pre = w->pre[l - 1];
+        ga.act = w->gl[l - 1];
+        if ((rc = gemm<wsn::EPI_GELU_BWD, true>(w, ga, st))) return rc;
+    }
+    // dW = act^T g and db = column sums of g, the batch in splits of at least 128 rows
+    int chunk = (batch + w->max_splits - 1) / w->max_splits;
+    chunk = std::max(128, (chunk + wsn::TK - 1) / wsn::TK * wsn::TK);
+    const int splits = (batch + chunk - 1) / chunk;
+    for (int l0 = 0; l0 < L; l0 += wsn::kGroup) {
+        wsn::WgradGroup q{};
+        q.layers = std::min(L - l0, wsn::kGroup);
+        q.chunk = chunk;
+        q.stride = w->nparams;
+        q.part = splits == 1 ? grad : w->part;
+        for (int k = 0; k < q.layers; ++k) {
+            const int l = l0 + k, in = w->sizes[l], out = w->sizes[l + 1];
+            q.g[k] = operands(w->act[l], in, w->gl[l], out);
+            q.g[k].M = in; q.g[k].N = out; q.g[k].K = batch;
+            q.woff[k] = w->w_off[l];
+            q.boff[k] = w->b_off[l];
+            q.tile0[k + 1] = q.tile0[k] + (in + wsn::TM - 1) / wsn::TM * ((out + wsn::TN - 1) / wsn::TN);
         }
+        wsn::wgrad_kernel<<<dim3(q.tile0[q.layers], splits), 128, 0, st>>>(q);
+        WCK(cudaGetLastError(), "weight gradient launch");
+    }
+    if (splits > 1) {
+        wsn::grad_reduce_kernel<<<grid_for(w->nparams), 256, 0, st>>>(w->part, w->nparams, splits, grad,
+                                                                       w->nparams);
+        WCK(cudaGetLastError(), "gradient reduction launch");
     }
     return SIM_OK;
 }
