@@ -671,14 +671,4 @@ __global__ void __launch_bounds__(SUBADMM_THREADS, 2) grid_step_kernel(StepParam
     if (pend) drain_stages(stage_bar[wl], &pend, &ph, nst);
 }
 
-// Self-test of the barrier's time limit: every block waits once for `expected` arrivals and
-// counts itself in `passed` when the wait ends (expected > blocks: nothing completes the
-// barrier, so every wait runs out and raises the error flag).
-__global__ void barrier_probe_kernel(unsigned *count, unsigned *gen, int *err, unsigned expected,
-                                     unsigned long long limit_ns, int *passed)
-{
-    grid_barrier(count, gen, err, expected, limit_ns);
-    if (threadIdx.x == 0) atomicAdd(passed, 1);
-}
-
 }  // namespace subadmm

@@ -1,6 +1,13 @@
 // Device-side description of a batch of scenes, built once by the host runtime when the
 // topology is fixed and read by the step kernel.  Internal to libsubadmm.
 #pragma once
+#include <cstddef>
+
+#ifdef __CUDACC__
+#define SUBADMM_HD __host__ __device__
+#else
+#define SUBADMM_HD
+#endif
 
 #define SUBADMM_MAXS 8          // most sides one constraint may have (|S_j|)
 #define SUBADMM_THREADS 256     // threads of one scene's block
@@ -9,6 +16,8 @@
 #define SUBADMM_MAXWARPS (SUBADMM_WIDE / 32)
 #define SUBADMM_MAXN 2048       // largest subsystem DOF
 #define SUBADMM_MAXM 2048       // largest side-row count of one subsystem
+#define SUBADMM_ITER 512        // threads of the grid's iteration kernel (one block per SM)
+#define SUBADMM_BIG 96          // grid kernel: DOF from which a block solves a subsystem
 #define SUBADMM_PARAMS 23       // doubles of a rigid-model constraint's parameters
 #define SUBADMM_BODY 17         // doubles of a body record
 
@@ -49,6 +58,9 @@ struct SceneDesc {
     int pre_off;
     int ord_off;           // ipool offset: the subsystems in decreasing order of per-warp setup
                            // work (the order the per-warp loops take them in)
+    int big_off, nbig;     // grid kernel: ipool offset and count of the subsystems of at least
+                           // SUBADMM_BIG DOF, which a whole block takes in the single-vector
+                           // solves
     int sr_g0, row_g0;     // global offset of the scene's side-rows / rows (z, lambda state)
     // double region
     int od_beta;           // beta per subsystem
@@ -128,6 +140,22 @@ struct GridScratch {
     double tsum;                   // exit residuals: theta, max |x - z|, max beta |dz| (bits)
     unsigned long long pmax, dmax;
     unsigned long long chk;        // mixed form: FP64 max |J v - z| (bits)
+    unsigned long long bar[2];     // iteration kernel: its barrier (arrivals, blocks not done)
+};
+
+// One warp's share of the grid's iteration kernel: a wave of whole projection items, at most
+// one side-row per lane, the rows of one subsystem on neighbouring lanes.
+struct WaveLane {
+    int t;                 // scene-local side-row (-1: idle)
+    int meta;              // type | row of its contact << 2 | writes lambda << 4 | sides << 5
+    int base, base2;       // lane of each side's first row, 5 bits per side (6 sides, then 2)
+};
+struct WaveHead {
+    unsigned starts;       // bit k: a batch (at most 8 rows of one subsystem) starts at lane k
+    int nrows;
+    int flags;             // 1: shape B (see grid_iter.cuh); 2: holds a contact; most sides of
+                           // an item << 8
+    int pad;
 };
 
 struct StepParams {
@@ -173,9 +201,51 @@ struct StepParams {
     GridScratch *grid;     // grid kernel scratch
     int grid_stage;        // grid kernel: bytes per staged D row in shared memory (filled
                            // by bulk copies), 0: rows read directly
+    const WaveLane *wave_lane;   // iteration kernel: 32 per wave
+    const WaveHead *wave_head;   // and their heads
+    int nwaves, wave_per_block;  // waves, and how many warps of a block take one
+    unsigned *wave_tag;    // iteration kernel: the tagged exchange's count, then its two buffers
+                           // from 16 bytes on (NULL: w through W0, W1 and the barrier)
+    int wave_smem;         // bytes of shared memory a warp may keep D rows in for the step
+    int tables;            // setup kernel: 1 to build the scene's tables (its first launch)
+    int grid_big;          // grid kernel: 1 if its shared memory holds the block solves of the
+                           // subsystems of at least SUBADMM_BIG DOF
     int grid_nstage;       // grid kernel: staged rows per warp (2 to 4)
     int nscenes;           // scenes of this launch
     int n_steps;
     double h, g0, g1, g2, gamma, rho, tol, theta_th;
     int beta_fixed, warm_prev, stop_theta, max_iters;
 };
+
+namespace subadmm {
+
+// Block solves of the grid kernel (block_solve.cuh): panels of 32 rows
+constexpr int kPanel = 32;
+constexpr int kTileLd = kPanel + 1;
+
+// shared memory that the block solves of a subsystem of n DOF and ngrp row groups take: the
+// groups' first rows and spans, then a BlockSolve of the wider type
+SUBADMM_HD inline size_t block_solve_groups(int ngrp) { return (size_t)(3 * ngrp + 4) * 4 / 16 * 16 + 16; }
+SUBADMM_HD inline size_t block_solve_bytes(int n, int ngrp)
+{
+    return block_solve_groups(ngrp) + 8 * ((size_t)(n + 1) / 2 * 2 + 2 * kPanel * kTileLd) + 4 * (size_t)n;
+}
+
+// Vectors (16 bytes) per lane of a wide row in a wave of shape B: 256 side-rows of a subsystem
+template <typename T>
+SUBADMM_HD constexpr int kWideVecs() { return sizeof(T) == 4 ? 2 : 4; }
+
+using KernFn = void (*)(StepParams);
+
+// The kernel variants, each instantiated in a translation unit of its own (they compile in
+// parallel): a scene per block, or one scene over the grid; FP32 or FP64 iterations
+KernFn block_kernel_f32(bool cached, int split, int nt);
+KernFn block_kernel_f64(bool cached, int split, int nt);
+KernFn grid_kernel_f32(int split);
+KernFn grid_kernel_f64(int split);
+KernFn grid_setup_f32();
+KernFn grid_setup_f64();
+KernFn grid_iter_f32(bool wide_rows);
+KernFn grid_iter_f64(bool wide_rows);
+
+}  // namespace subadmm

@@ -111,7 +111,7 @@ __device__ __forceinline__ void side_row(const Side &s, const double *dir, const
 
 // Rows of a model constraint: Ja, Jb are rows x 6 blocks of sides a and b (a node side
 // uses the first 3 columns), e the error terms; k, alpha (soft) are returned for ANGLE_PD.
-__device__ void model_rows(const ConDesc &c, const double *prm, const double *bodies,
+static __device__ void model_rows(const ConDesc &c, const double *prm, const double *bodies,
                            const double *nodes, double h, double gamma, double *Ja, double *Jb,
                            double *e, double *k_out, double *alpha_out)
 {
@@ -283,7 +283,7 @@ __device__ __forceinline__ void inv3_cof(const double *M, double *c, double &det
     det = M[0] * c[0] + M[1] * c[1] + M[2] * c[2];
 }
 
-__device__ void corot_element(const int *tet, const double *Ke, const double *X0,
+static __device__ void corot_element(const int *tet, const double *Ke, const double *X0,
                               const double *nodes, double h, int n, double *K, double *b)
 {
     double Dm[9], Ds[9];

@@ -36,6 +36,7 @@
 #pragma once
 #include "layout.h"
 #include "rigid_model.cuh"
+#include "block_solve.cuh"
 
 namespace subadmm {
 
@@ -205,7 +206,8 @@ struct BlockDist {
     // chunks of W wait on per-subsystem flags instead of a barrier after the factor loop (a
     // scene over the whole grid has far more warps than subsystems, and its pollers would
     // load the L2 that its factorisations run through)
-    static constexpr bool kSpread = true;
+    static constexpr bool kSpread = true, kBig = false;
+    static constexpr int kThreads = SUBADMM_THREADS;
     int tid, nthreads, warp, nwarps;
     __device__ __forceinline__ BlockDist()
         : tid(threadIdx.x), nthreads(blockDim.x), warp(threadIdx.x >> 5), nwarps(blockDim.x >> 5) {}
@@ -228,7 +230,7 @@ __device__ __forceinline__ unsigned long long global_ns()
 // wait longer than limit_ns, or an error raised by another block, sets / sees the error
 // flag and returns at once, here and at every later barrier, so the grid always runs to its
 // end.  (`gen` is unused: kept for the scratch layout.)
-__device__ __noinline__ void grid_barrier(unsigned *count, unsigned *gen, int *err,
+static __device__ __noinline__ void grid_barrier(unsigned *count, unsigned *gen, int *err,
                                           unsigned expected, unsigned long long limit_ns)
 {
     (void)gen;
@@ -258,7 +260,8 @@ __device__ __noinline__ void grid_barrier(unsigned *count, unsigned *gen, int *e
 // work (one warp each, FP64-bound in the setup and the recovery) then spreads over one warp
 // per block, i.e. over the SMs and their FP64 pipes, instead of filling the first blocks.
 struct GridDist {
-    static constexpr bool kSpread = false;
+    static constexpr bool kSpread = false, kBig = false;
+    static constexpr int kThreads = SUBADMM_THREADS;
     int tid, nthreads, warp, nwarps;
     unsigned *count, *gen;
     int *err;
@@ -696,7 +699,8 @@ __device__ void w_chunks(const StepParams &P, const SceneDesc &S, const View<T> 
 // assemble .. factor .. map, and the per-step constants of the z-step
 template <typename T, typename Dist>
 __device__ long long scene_setup(const StepParams &P, const SceneDesc &S, const View<T> &V,
-                                 int *s_status, int step, const Dist &d)
+                                 int *s_status, int step, const Dist &d,
+                                 unsigned char *big_smem = nullptr)
 {
     const int lane = threadIdx.x & 31;
     constexpr bool MIXED = sizeof(T) == 4;
@@ -848,10 +852,45 @@ __device__ long long scene_setup(const StepParams &P, const SceneDesc &S, const 
     // the map W = L^-1 [J^T b], D = W^T W, c.  The FP64 form and the stiff blocks of the mixed
     // form factorise K in FP64 (rounded into the T copy); the other mixed blocks factorise in
     // FP32, keeping the FP64 A, b and J for the recovery and refinement of v-hat.
+    if constexpr (!Dist::kSpread) {
+        // the large subsystems whose factor is kept, a block each: c = J K^-1 b from one solve
+        // and J's spans (two solves of the vector instead of g = L^-1 b and a pass over the
+        // whole of W, 3 MB a slab: 3.6M -> 0.63M SM cycles for 64 slabs); the flag 0 then
+        // leaves nothing to the passes below
+        for (int k = blockIdx.x; big_smem && k < S.nbig; k += gridDim.x) {
+            const int i = P.ipool[S.big_off + k], gsub = S.sub0 + i;
+            const SubDesc &u = P.subs[gsub];
+            if (!factor_kept(P, S, u, gsub, step)) continue;
+            const SubEnv e = sub_env(P, u);
+            const int n = u.n;
+            const double *b = sdb + u.od_b, *J = sdb + u.od_J;
+            const T *LT = stb + u.ot_L;
+            T *cc = htb + u.ot_c;
+            BlockSolve<T> bs(big_smem, n);
+            for (int p = threadIdx.x; p < n; p += Dist::kThreads) bs.x[p] = (T)b[p];
+            block_solve_begin<Dist::kThreads>(LT, n, e.env, bs);
+            block_forward<Dist::kThreads, T, true>(LT, nullptr, n, e.lastr, bs);
+            block_backward<Dist::kThreads, T, true>(LT, nullptr, n, bs);
+            for (int r = threadIdx.x; r < u.m; r += Dist::kThreads) {
+                T acc = (T)0;
+                for (int p = e.jlo[r]; p < e.jhi[r]; ++p) acc += (T)J[(size_t)r * n + p] * bs.x[p];
+                cc[r] = acc;
+            }
+            if (threadIdx.x == 0) {
+                if (step == 0) {
+                    db[S.od_beta + i] = P.beta[gsub];
+                    db[S.od_flag + i] = (P.subflag[gsub] & 2) ? 1.0 : 0.0;
+                }
+                P.pending[gsub] = 0;
+            }
+            __syncthreads();
+        }
+    }
     for (int k = d.warp; k < S.nsub; k += d.nwarps) {
         const int i = Dist::kSpread ? __ldg(P.ipool + S.ord_off + k) : k;   // largest first
         const SubDesc &u = P.subs[S.sub0 + i];
         const int gsub = S.sub0 + i;
+        if (!Dist::kSpread && big_smem && u.n >= SUBADMM_BIG && factor_kept(P, S, u, gsub, step)) continue;
         // W's leading dimension: m + 1 columns rounded up to 4 (map_item reads 4-column blocks)
         const int n = u.n, m = u.m, ldw = (m + 1 + 3) / 4 * 4;
         const SubEnv e = sub_env(P, u);
@@ -1108,6 +1147,101 @@ __device__ __forceinline__ void warp_chol_solve(const T *LT, T *s, int n, const 
     }
 }
 
+// J^T w of one column p (FP64): the row groups that hold it in order, each summed over its rows
+// before it is added (the arithmetic of add_jt); grp: the groups' first rows and column spans
+template <typename W>
+__device__ __forceinline__ double column_jt(double out, const double *J, int n, int p, int ngrp,
+                                            const int *grp, const W *w)
+{
+    for (int g = 0; g < ngrp; ++g) {
+        if (p < grp[3 * g + 1] || p >= grp[3 * g + 2]) continue;
+        double acc = 0.0;
+        for (int r = grp[3 * g]; r < grp[3 * g + 3]; ++r) acc += J[(size_t)r * n + p] * (double)w[r];
+        out += acc;
+    }
+    return out;
+}
+
+// v-hat of one subsystem by a whole block (see recover_v): the vector and the row groups'
+// spans in shared memory, the solves of block_solve.cuh.  A linear block's A is read through
+// K's sparse pattern (45 entries a row where the band holds 270).  1200-DOF slabs, the exit phase:
+// FP32 factor with refinement 10.6M -> 2.2M SM cycles, FP64 factor 5.0M -> 1.5M.
+template <typename T, int NT>
+__device__ __noinline__ void block_recover_one(const StepParams &P, const SceneDesc &S, const View<T> &V,
+                                               const T *w, int i, unsigned char *smem)
+{
+    constexpr bool MIXED = sizeof(T) == 4;
+    const SubDesc &u = P.subs[S.sub0 + i];
+    const int n = u.n, m = u.m, tid = threadIdx.x;
+    const SubEnv e = sub_env(P, u);
+    const double *J = V.sdb + u.od_J, *Lf = V.sdb + u.od_L, *b = V.sdb + u.od_b;
+    double *idg = V.sdb + u.od_id, *v = V.sdb + u.od_v;
+    const T *wi = w + u.sr0;
+    int *grp = reinterpret_cast<int *>(smem);
+    smem += block_solve_groups(e.ngrp);
+    for (int g = tid; g <= e.ngrp; g += NT) {
+        grp[3 * g] = e.grp[g];
+        if (g < e.ngrp) { grp[3 * g + 1] = e.jlo[e.grp[g]]; grp[3 * g + 2] = e.jhi[e.grp[g]]; }
+    }
+    __syncthreads();
+    if (!MIXED || V.db[S.od_flag + i] != 0.0) {
+        BlockSolve<double> s(smem, n);
+        for (int p = tid; p < n; p += NT)
+            s.x[p] = column_jt(b[p], J, n, p, e.ngrp, grp, wi);
+        __syncthreads();
+        block_solve_begin<NT>(Lf, n, e.env, s);
+        block_forward<NT, double, false>(Lf, idg, n, e.lastr, s);
+        block_backward<NT, double, false>(Lf, idg, n, s);
+        for (int p = tid; p < n; p += NT) v[p] = s.x[p];
+        __syncthreads();
+        return;
+    }
+    BlockSolve<T> s(smem, n);
+    const T *LT = V.stb + u.ot_L;
+    block_solve_begin<NT>(LT, n, e.env, s);
+    double *rhs = idg, *t = V.sdb + u.od_t;
+    const double beta = V.db[S.od_beta + i];
+    for (int p = tid; p < n; p += NT) {
+        rhs[p] = column_jt(b[p], J, n, p, e.ngrp, grp, wi);
+        s.x[p] = (T)rhs[p];
+    }
+    __syncthreads();
+    block_forward<NT, T, true>(LT, nullptr, n, e.lastr, s);
+    block_backward<NT, T, true>(LT, nullptr, n, s);
+    for (int p = tid; p < n; p += NT) v[p] = (double)s.x[p];
+    __syncthreads();
+    for (int r = tid; r < m; r += NT) {
+        double acc = 0.0;
+        for (int p = e.jlo[r]; p < e.jhi[r]; ++p) acc += J[(size_t)r * n + p] * v[p];
+        t[r] = acc * -beta;
+    }
+    __syncthreads();
+    const int *rowp = P.ipool + u.csr_off, *col = rowp + n + 1;
+    for (int p = tid; p < n; p += NT) {
+        double acc = column_jt(rhs[p], J, n, p, e.ngrp, grp, t);
+        const double *Ap = Lf + (size_t)p * n;
+        if (u.kind == KIND_LINEAR) {
+            bool diag = false;                    // (K's pattern may leave a diagonal entry out)
+            for (int q = rowp[p]; q < rowp[p + 1]; ++q) {
+                const int c = col[q];
+                diag = diag || c == p;
+                acc -= Ap[c] * v[c];
+            }
+            if (!diag) acc -= Ap[p] * v[p];
+        } else if (u.kind == KIND_RIGID) {
+            acc -= Ap[p] * v[p];                  // A is diagonal
+        } else {
+            for (int q = e.env[p]; q <= e.lastr[p]; ++q) acc -= Ap[q] * v[q];
+        }
+        s.x[p] = (T)acc;
+    }
+    __syncthreads();
+    block_forward<NT, T, true>(LT, nullptr, n, e.lastr, s);
+    block_backward<NT, T, true>(LT, nullptr, n, s);
+    for (int p = tid; p < n; p += NT) v[p] += (double)s.x[p];
+    __syncthreads();
+}
+
 // v-hat of the last v-step, v = K^-1 (b + J^T w), in FP64 (warp per subsystem) into od_v.
 // With an FP64 factor (FP64 form, or a stiff block of the mixed form): two triangular
 // solves.  With an FP32 factor: a solve, then one step of iterative refinement with the
@@ -1115,15 +1249,24 @@ __device__ __forceinline__ void warp_chol_solve(const T *LT, T *s, int n, const 
 // K v = A v + beta J^T (J v).
 // `fast` (may be null): per-warp shared memory of fast_len T values; the FP32 solves of a
 // subsystem with n <= fast_len run on a copy there instead of on the global scratch vector.
+// `big_smem` (may be null): shared memory of this block in which it solves the subsystems of at
+// least SUBADMM_BIG DOF, a block per subsystem; the others go to the warps, from the last
+// block on (the first blocks hold the large ones).
 template <typename T, typename Dist>
 __device__ void recover_v(const StepParams &P, const SceneDesc &S, const View<T> &V, const T *w,
-                          const Dist &d, T *fast = nullptr, int fast_len = 0)
+                          const Dist &d, T *fast = nullptr, int fast_len = 0,
+                          unsigned char *big_smem = nullptr)
 {
     constexpr bool MIXED = sizeof(T) == 4;
     const int lane = threadIdx.x & 31;
-    for (int k = d.warp; k < S.nsub; k += d.nwarps) {
+    if constexpr (Dist::kBig)                     // (grid_iter.cuh)
+        for (int k = blockIdx.x; big_smem && k < S.nbig; k += gridDim.x)
+            block_recover_one<T, Dist::kThreads>(P, S, V, w, P.ipool[S.big_off + k], big_smem);
+    const int w0 = Dist::kSpread || !big_smem ? d.warp : d.nwarps - 1 - d.warp;
+    for (int k = w0; k < S.nsub; k += d.nwarps) {
         const int i = Dist::kSpread ? __ldg(P.ipool + S.ord_off + k) : k;   // largest first
         const SubDesc &u = P.subs[S.sub0 + i];
+        if (big_smem && u.n >= SUBADMM_BIG) continue;
         const int n = u.n, m = u.m;
         const SubEnv e = sub_env(P, u);
         // od_L holds the FP64 factor L (FP64 form) or A itself (mixed form)

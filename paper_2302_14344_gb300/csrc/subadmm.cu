@@ -15,12 +15,13 @@
 #include "subadmm.h"
 #include "layout.h"
 #include "step_kernel.cuh"
-#include "grid_kernel.cuh"
 #include "features.cuh"
 #include "warmstart.h"
 #include "device_guard.h"
 #include "gram.h"
 #include "chol.h"
+
+using subadmm::KernFn;
 
 namespace {
 
@@ -55,6 +56,18 @@ struct LaunchClass {
     int max_smem = 0;
     cudaStream_t stream = nullptr; // class 0 runs on the simulation's stream
     cudaEvent_t done = nullptr;
+};
+
+// A grid scene's layout for the iteration kernel (grid_iter.cuh), for one block count
+struct IterPlan {
+    int blocks = 0;                // the count it was built for (0: not built)
+    int nwaves = 0, per_block = 0; // nwaves 0: the scene has more side-rows than lanes
+    bool wide = false;             // rows too wide for shared memory slots: the LONG kernel
+    int row_share = 0;             // shared memory of a warp: its slots, or (LONG) the most bytes of
+                                   // D rows of a wave
+    unsigned *d_tag = nullptr;     // the tagged exchange (not LONG)
+    WaveLane *d_lane = nullptr;
+    WaveHead *d_head = nullptr;
 };
 
 struct HostCon {
@@ -109,6 +122,7 @@ struct sim_s {
     cudaEvent_t ev_fork = nullptr;
     int split_override = 0;        // tuning: force the split of every class (0: heuristic)
     std::vector<int> sc_nsr, sc_items, sc_sides, sc_mpad;   // per scene: register-cache limits
+    std::vector<int> sc_big;       // per scene: shared memory of the grid kernel's block solves
     std::vector<int> sc_fmap_ok;   // per scene: bit si set if the thread map for 2^si lanes exists
     int smem_full = 0;             // dynamic shared memory a block may use
     int grid_side_rows = kGridSideRows;
@@ -123,6 +137,10 @@ struct sim_s {
                                    // Cholesky with tensor-core Schur updates
     std::vector<subadmm::CholPlan> chol;   // per scene: the blocked factorisation's panels
     std::vector<int> h_ipool;      // host copy of the integer pool (envelopes)
+    std::vector<IterPlan> iter;            // per scene: grid scenes' iteration layout
+    std::vector<char> grid_tables;         // per scene: its tables are in the workspace
+    std::vector<Item> h_items;             // host copies of the projection items
+    std::vector<int> h_lists;
     std::vector<char> grid_factored;       // per scene: its tc subsystems hold kept factors
     // graph replay of sim_step
     bool use_graph = false;
@@ -281,6 +299,9 @@ void free_device(sim_t s)
     for (auto &c : s->chol) subadmm::chol_plan_free(c);
     s->chol.clear();
     s->grid_factored.clear();
+    for (auto &p : s->iter) { cudaFree(p.d_lane); cudaFree(p.d_head); cudaFree(p.d_tag); }
+    s->iter.clear();
+    s->grid_tables.clear();
     if (s->graph_stream) cudaStreamDestroy(s->graph_stream);
     s->graph_stream = nullptr;
     s->d_nodes = nullptr; s->d_ipool = nullptr; s->d_subflag = nullptr;
@@ -310,6 +331,9 @@ int zeros(sim_t s, double **dst, size_t count, const char *what)
     if (e != cudaSuccess) return cuda_fail(s, e, what);
     return SIM_OK;
 }
+
+int iter_blocks(const sim_t s, int sms, int div);
+int iter_plan_of(sim_t s, int sc, int blocks);
 
 // Lays out every scene for the step kernel and uploads it.
 int finalize(sim_t s)
@@ -352,6 +376,8 @@ int finalize(sim_t s)
     int max_nsr = 0, max_items = 0, max_sides = 0, max_mpad = 0;
     struct Place { long long sd, st, sh, scd, scene_t, ints; };
     std::vector<Place> place(nscenes);
+    std::vector<int> &sc_big = s->sc_big;
+    sc_big.assign(nscenes, 0);
     std::vector<int> sc_mpad(nscenes, 0), sc_sides(nscenes, 0), sc_fmap_ok(nscenes, 0);
     s->sdesc.assign(nsubs, SubDesc{});
     s->cdesc.assign(ncons, ConDesc{});
@@ -578,6 +604,17 @@ int finalize(sim_t s)
             std::stable_sort(ord.begin(), ord.end(),
                              [&](int a, int b) { return setup_cost[a] > setup_cost[b]; });
             ipool.insert(ipool.end(), ord.begin(), ord.end());
+        }
+        // the subsystems that a block takes in the grid kernel's single-vector solves
+        S.big_off = (int)ipool.size();
+        S.nbig = 0;
+        sc_big[sc] = 0;
+        for (int i = 0; i < S.nsub; ++i) {
+            const SubDesc &u = s->sdesc[S.sub0 + i];
+            if (u.n < SUBADMM_BIG) continue;
+            ipool.push_back(i);
+            ++S.nbig;
+            sc_big[sc] = std::max(sc_big[sc], (int)subadmm::block_solve_bytes(u.n, u.ngrp));
         }
         // work of the setup's scene-wide passes, as prefix sums over the scene's subsystems:
         // chunks of 32 columns of W = L^-1 [J^T b] (m + 1 columns), then the map's items of
@@ -927,6 +964,10 @@ int finalize(sim_t s)
     if ((rc = upload(s, &s->d_nodes, nodes, "nodes"))) return rc;
     if ((rc = upload(s, &s->d_ipool, ipool, "integer pool"))) return rc;
     s->h_ipool = ipool;
+    s->h_items = items;
+    s->h_lists = lists;
+    s->iter.assign(nscenes, IterPlan{});
+    s->grid_tables.assign(nscenes, 0);
     {
         {
             const std::vector<double> ones(std::max(1, nsubs), 1.0);
@@ -958,6 +999,13 @@ int finalize(sim_t s)
         cudaError_t e = cudaMalloc((void **)&s->d_stats, std::max(1, 5 * nscenes) * sizeof(long long));
         if (e != cudaSuccess) return fail(s, SIM_ENOMEM, "cudaMalloc stats");
         CK(cudaMemsetAsync(s->d_stats, 0, std::max(1, 5 * nscenes) * sizeof(long long), s->stream), "memset stats");
+    }
+    if (s->opt.stop != SIM_STOP_THETA) {
+        int sms = 0;
+        CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->opt.device), "attribute");
+        for (const LaunchClass &c : s->classes)
+            for (int sc : c.scenes)
+                if (c.grid && (rc = iter_plan_of(s, sc, iter_blocks(s, sms, c.block_div)))) return rc;
     }
     s->finalized = true;
     return SIM_OK;
@@ -1227,7 +1275,15 @@ int sim_set_generic(sim_t s, int sub, const double *A, const double *b)
 
 namespace {
 
-using KernFn = void (*)(StepParams);
+// Self-test of the barrier's time limit: every block waits once for `expected` arrivals and
+// counts itself in `passed` when the wait ends (expected > blocks: nothing completes the
+// barrier, so every wait runs out and raises the error flag).
+__global__ void barrier_probe_kernel(unsigned *count, unsigned *gen, int *err, unsigned expected,
+                                     unsigned long long limit_ns, int *passed)
+{
+    subadmm::grid_barrier(count, gen, err, expected, limit_ns);
+    if (threadIdx.x == 0) atomicAdd(passed, 1);
+}
 
 // `iters` rounds of the block barrier that ends every iteration of the block kernel
 // (__syncthreads_count), with nothing else between them: the floor of one iteration
@@ -1274,6 +1330,14 @@ StepParams step_params(const sim_t s, int n_steps)
     P.scene_ids = s->d_scene_ids;
     P.grid = s->d_grid;
     P.lam0 = nullptr;
+    P.grid_stage = 0;
+    P.grid_nstage = 0;
+    P.wave_lane = nullptr;
+    P.wave_head = nullptr;
+    P.wave_tag = nullptr;
+    P.nwaves = P.wave_per_block = P.wave_smem = 0;
+    P.tables = 1;
+    P.grid_big = 0;
     P.tc_phase = 0;
     P.tc_factor = 0;
     P.ref10 = s->d_ref10;
@@ -1283,29 +1347,12 @@ StepParams step_params(const sim_t s, int n_steps)
 
 KernFn kernel_for(bool mixed, bool cached, int split, int nt = SUBADMM_THREADS)
 {
-    using namespace subadmm;
-    if (!cached && nt == SUBADMM_WIDE) {
-        if (mixed)
-            return split == 4 ? step_kernel<float, 4, false, SUBADMM_WIDE>
-                 : split == 2 ? step_kernel<float, 2, false, SUBADMM_WIDE>
-                              : step_kernel<float, 1, false, SUBADMM_WIDE>;
-        return split == 4 ? step_kernel<double, 4, false, SUBADMM_WIDE>
-             : split == 2 ? step_kernel<double, 2, false, SUBADMM_WIDE>
-                          : step_kernel<double, 1, false, SUBADMM_WIDE>;
-    }
-    if (mixed) {
-        if (cached) return split == 4 ? step_kernel<float, 4, true> : split == 2 ? step_kernel<float, 2, true> : step_kernel<float, 1, true>;
-        return split == 4 ? step_kernel<float, 4, false> : split == 2 ? step_kernel<float, 2, false> : step_kernel<float, 1, false>;
-    }
-    if (cached) return split == 4 ? step_kernel<double, 4, true> : split == 2 ? step_kernel<double, 2, true> : step_kernel<double, 1, true>;
-    return split == 4 ? step_kernel<double, 4, false> : split == 2 ? step_kernel<double, 2, false> : step_kernel<double, 1, false>;
+    return mixed ? subadmm::block_kernel_f32(cached, split, nt) : subadmm::block_kernel_f64(cached, split, nt);
 }
 
 KernFn grid_kernel_for(bool mixed, int split)
 {
-    using namespace subadmm;
-    if (mixed) return split == 32 ? grid_step_kernel<float, 32> : split == 16 ? grid_step_kernel<float, 16> : grid_step_kernel<float, 8>;
-    return split == 32 ? grid_step_kernel<double, 32> : split == 16 ? grid_step_kernel<double, 16> : grid_step_kernel<double, 8>;
+    return mixed ? subadmm::grid_kernel_f32(split) : subadmm::grid_kernel_f64(split);
 }
 
 // One cooperative launch per scene of a grid class, in turn on `st`, each after zeroing the
@@ -1373,6 +1420,270 @@ int chol_plan_of(sim_t s, int sc)
     return SIM_OK;
 }
 
+// Blocks of the iteration kernel: one per SM, fewer if the caller fixed the count
+int iter_blocks(const sim_t s, int sms, int div)
+{
+    return s->grid_blocks > 0 ? std::min(s->grid_blocks, sms) : std::max(1, sms / std::max(1, div));
+}
+
+// Lays out the waves of grid scene sc over `blocks` blocks: the projection items sorted by the
+// subsystems they join, cut into runs of nearly equal work (vectors of D, plus a constant per
+// row), whole items, at most 32 side-rows.  A wave is short when it has at most 8 rows of at
+// most 32 vectors (one per lane): as long as there are warps enough, runs are cut there.
+int iter_plan_of(sim_t s, int sc, int blocks)
+{
+    if (s->iter[sc].blocks == blocks) return SIM_OK;
+    const SceneDesc &S = s->scenes[sc];
+    const int vn = s->opt.precision == SIM_MIXED ? 4 : 2, warps = blocks * (SUBADMM_ITER / 32);
+    std::vector<int> sub(S.nsr, 0);                  // subsystem of each side-row
+    for (int i = 0; i < S.nsub; ++i) {
+        const SubDesc &u = s->sdesc[S.sub0 + i];
+        for (int r = 0; r < u.m; ++r) sub[u.sr0 + r] = i;
+    }
+    auto vecs = [&](int t) { return (s->sdesc[S.sub0 + sub[t]].m + vn - 1) / vn; };
+    const int rv = vn == 4 ? subadmm::kWideVecs<float>() : subadmm::kWideVecs<double>();
+    // an item: its subsystems, rows, and how many of those are wide (more than 32 vectors); it
+    // fits the slots if at most 3 are, of one subsystem, of at most 32 rv vectors
+    struct Work { int item, a, b, rows, wide, wsub; bool fits; long long cost; };
+    std::vector<Work> work;
+    long long total = 0;
+    bool slots = true;
+    for (int k = 0; k < S.nitem; ++k) {
+        const Item &I = s->h_items[S.item_g0 + k];
+        if (I.type < 0) continue;
+        const int nr = I.type == TYPE_CONTACT ? 3 : 1;
+        const int *ls = s->h_lists.data() + S.list_g0 + I.lo;
+        Work w{k, sub[ls[0]], I.ns > 1 ? sub[ls[1]] : -1, I.ns * nr, 0, -1, true, 0};
+        if (w.a > w.b && w.b >= 0) std::swap(w.a, w.b);
+        for (int q = 0; q < I.ns; ++q) {
+            const int v = vecs(ls[q]);
+            w.cost += (long long)nr * ((v + 31) / 32 * 32 + 16);
+            if (v <= 32) continue;
+            w.fits = w.fits && v <= 32 * rv && (w.wsub < 0 || w.wsub == sub[ls[q]]);
+            w.wide += nr;
+            w.wsub = sub[ls[q]];
+        }
+        w.fits = w.fits && w.wide <= 3 && w.rows - w.wide <= (w.wide ? 3 : 8);
+        slots = slots && w.fits;
+        total += w.cost;
+        work.push_back(w);
+    }
+    // (items with wide rows in waves of their own, by the wide subsystem)
+    std::stable_sort(work.begin(), work.end(), [](const Work &p, const Work &q) {
+        return p.wsub != q.wsub ? p.wsub < q.wsub : p.a != q.a ? p.a < q.a : p.b < q.b;
+    });
+    std::vector<std::vector<int>> waves;             // indices into work
+    auto cut = [&](bool in_slots, double target) {
+        waves.clear();
+        int rows = 0, wide = 0;
+        long long cost = 0;
+        for (int k = 0; k < (int)work.size(); ++k) {
+            const Work &w = work[k];
+            const bool full = !in_slots ? rows + w.rows > 32
+                              : w.wide  ? wide + w.wide > 3 || rows - wide + w.rows - w.wide > 3
+                                        : rows + w.rows > 8;
+            if (k == 0 || full || cost + w.cost / 2 > target || (in_slots && w.wsub != work[k - 1].wsub)) {
+                waves.emplace_back();
+                rows = wide = 0;
+                cost = 0;
+            }
+            waves.back().push_back(k);
+            rows += w.rows;
+            wide += w.wide;
+            cost += w.cost;
+        }
+        return (int)waves.size() <= warps;
+    };
+    bool ok = false;
+    const double even = (double)total / warps;
+    for (double f = 1.0; slots && !ok && f < 4.0; f *= 1.05) ok = cut(true, f * even);
+    const bool in_slots = ok;
+    for (double f = 1.0; !ok && f < 8.0; f *= 1.05) ok = cut(false, f * even);
+    IterPlan P;
+    P.blocks = blocks;
+    std::vector<WaveLane> lane;
+    std::vector<WaveHead> head;
+    if (ok) {
+        P.nwaves = (int)waves.size();
+        P.wide = !in_slots;
+        P.per_block = std::max(1, (P.nwaves + blocks - 1) / blocks);
+        for (const auto &wv : waves) {
+            struct Row { int t, item, side, r; };
+            std::vector<Row> rows;
+            for (int k : wv) {
+                const Item &I = s->h_items[S.item_g0 + work[k].item];
+                const int nr = I.type == TYPE_CONTACT ? 3 : 1;
+                for (int q = 0; q < I.ns; ++q)
+                    for (int r = 0; r < nr; ++r)
+                        rows.push_back({s->h_lists[S.list_g0 + I.lo + q] + r, work[k].item, q, r});
+            }
+            // rows of one subsystem side by side (an item's side stays together)
+            // (shape B: the wide rows first, the narrow ones from lane 3 on)
+            std::stable_sort(rows.begin(), rows.end(), [&](const Row &p, const Row &q) {
+                const bool wp = in_slots && vecs(p.t) > 32, wq = in_slots && vecs(q.t) > 32;
+                return wp != wq ? wp : sub[p.t] < sub[q.t];
+            });
+            const bool shape_b = in_slots && vecs(rows[0].t) > 32;
+            if (shape_b) {
+                size_t nwide = 0;
+                while (nwide < rows.size() && vecs(rows[nwide].t) > 32) ++nwide;
+                if (nwide < rows.size())
+                    while (nwide < 3) { rows.insert(rows.begin() + nwide, Row{-1, -1, 0, 0}); ++nwide; }
+            }
+            WaveHead H{0u, (int)rows.size(), 0, 0};
+            const size_t l0 = lane.size();
+            int most = 0, bytes = 0;
+            for (int k = 0; k < 32; ++k) lane.push_back(WaveLane{-1, 1 << 5, k, 0});
+            for (int k = 0, first = 0; k < (int)rows.size(); ++k) {
+                const Row &R = rows[k];
+                if (R.t < 0) { first = k; continue; }
+                const Item &I = s->h_items[S.item_g0 + R.item];
+                if (k == 0 || rows[k - 1].t < 0 || sub[R.t] != sub[rows[k - 1].t] || k - first == 8) { H.starts |= 1u << k; first = k; }
+                WaveLane &L = lane[l0 + k];
+                L.t = R.t;
+                L.meta = I.type | R.r << 2 | (R.side == 0 ? 16 : 0) | I.ns << 5;
+                L.base = L.base2 = 0;
+                for (int j = 0; j < (int)rows.size(); ++j) {
+                    if (rows[j].item != R.item || rows[j].r != 0) continue;
+                    if (rows[j].side < 6) L.base |= j << (5 * rows[j].side);
+                    else L.base2 |= j << (5 * (rows[j].side - 6));
+                }
+                most = std::max(most, I.ns);
+                if (I.type == TYPE_CONTACT) H.flags |= 2;
+                bytes += 16 * vecs(R.t);
+            }
+            H.flags |= (shape_b ? 1 : 0) | most << 8;
+            P.row_share = std::max(P.row_share, bytes);
+            head.push_back(H);
+        }
+    }
+    IterPlan &old = s->iter[sc];
+    if (old.d_lane) {
+        CK(cudaStreamSynchronize(s->stream), "iteration plan");     // launches that read the old one
+        cudaFree(old.d_lane);
+        cudaFree(old.d_head);
+        cudaFree(old.d_tag);
+        old = IterPlan{};
+    }
+    if (P.nwaves > 0) {
+        if (cudaMalloc((void **)&P.d_lane, lane.size() * sizeof(WaveLane)) != cudaSuccess)
+            return fail(s, SIM_ENOMEM, "cudaMalloc iteration plan");
+        old = P;
+        if (cudaMalloc((void **)&P.d_head, head.size() * sizeof(WaveHead)) != cudaSuccess) {
+            old.blocks = 0;
+            return fail(s, SIM_ENOMEM, "cudaMalloc iteration plan");
+        }
+        CK(cudaMemcpy(P.d_lane, lane.data(), lane.size() * sizeof(WaveLane), cudaMemcpyHostToDevice), "iteration plan");
+        old = P;
+        CK(cudaMemcpy(P.d_head, head.data(), head.size() * sizeof(WaveHead), cudaMemcpyHostToDevice), "iteration plan");
+        if (in_slots) {
+            P.row_share = 512 * std::max(8, 3 * rv + 3);
+            // the tagged words of every side-row, twice: tag 0x80000000 matches no iteration, ~0
+            // marks padding side-rows (no owner, value 0)
+            const int words = vn == 4 ? 2 : 4;
+            std::vector<unsigned> tags(4 + 2 * (size_t)S.nsr * words, 0u);
+            for (size_t t = 0; t < 2 * (size_t)S.nsr; ++t)
+                for (int k = 1; k < words; k += 2) tags[4 + t * words + k] = ~0u;
+            for (const WaveLane &L : lane)
+                for (int half = 0; half < 2 && L.t >= 0; ++half)
+                    for (int k = 1; k < words; k += 2)
+                        tags[4 + ((size_t)half * S.nsr + L.t) * words + k] = 0x80000000u;
+            if (cudaMalloc((void **)&P.d_tag, tags.size() * 4) != cudaSuccess)
+                return fail(s, SIM_ENOMEM, "cudaMalloc iteration plan");
+            old = P;
+            CK(cudaMemcpy(P.d_tag, tags.data(), tags.size() * 4, cudaMemcpyHostToDevice), "iteration plan");
+        }
+    }
+    s->iter[sc] = P;
+    return SIM_OK;
+}
+
+// A cooperative launch of `blocks` blocks with `dyn` bytes of shared memory
+int coop_launch(sim_t s, KernFn kf, int blocks, int threads, size_t dyn, StepParams &P, cudaStream_t st)
+{
+    CK(cudaFuncSetAttribute((const void *)kf, cudaFuncAttributeMaxDynamicSharedMemorySize, s->smem_full),
+       "shared memory attribute");
+    void *args[] = {&P};
+    CK(cudaLaunchCooperativeKernel((const void *)kf, dim3(blocks), dim3(threads), args, dyn, st), "grid kernel launch");
+    return SIM_OK;
+}
+
+// The steps of one grid scene as setup and iteration launches (grid_iter.cuh).
+int launch_grid_fused(sim_t s, LaunchClass &c, StepParams P, cudaStream_t st, int sc, bool capturing)
+{
+    const bool mixed = s->opt.precision == SIM_MIXED;
+    const SceneDesc &S = s->scenes[sc];
+    const IterPlan &plan = s->iter[sc];
+    const KernFn setup = mixed ? subadmm::grid_setup_f32() : subadmm::grid_setup_f64();
+    const KernFn iter = mixed ? subadmm::grid_iter_f32(plan.wide) : subadmm::grid_iter_f64(plan.wide);
+    // block solves of large subsystems: in the setup's shared memory if that leaves two blocks per
+    // SM, in the iteration kernel's (the whole SM's) next to nothing else
+    const int need = s->sc_big[sc];
+    const bool big = need > 0 && need <= s->smem_full / 2;
+    int per_sm = 0, sms = 0;
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->opt.device), "attribute");
+    CK(cudaFuncSetAttribute((const void *)setup, cudaFuncAttributeMaxDynamicSharedMemorySize, s->smem_full),
+       "shared memory attribute");
+    CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, setup, SUBADMM_THREADS, big ? need : 0), "occupancy");
+    const int resident = std::max(1, per_sm * sms);
+    const int blocks = s->grid_blocks > 0 ? std::min(s->grid_blocks, resident)
+                                          : std::max(1, resident / std::max(1, c.block_div));
+    const int warps = SUBADMM_ITER / 32;
+    const int share = !plan.wide ? plan.row_share
+                      : s->grid_staging ? std::min(plan.row_share, s->smem_full / warps / 16 * 16) : 0;
+    const size_t dyn = std::max<size_t>((size_t)share * warps, big ? need : 0);
+    c.max_smem = std::max(c.max_smem, share * warps);
+    const int n_steps = P.n_steps;
+    P.nscenes = 1;
+    P.n_steps = 1;
+    P.wave_lane = plan.d_lane;
+    P.wave_head = plan.d_head;
+    P.nwaves = plan.nwaves;
+    P.wave_per_block = plan.per_block;
+    P.wave_smem = share;
+    P.grid_big = big ? 1 : 0;
+    int rc = gram_plan_of(s, sc);
+    if (rc) return rc;
+    const bool blocked = s->tc_factor && s->gram[sc].njobs > 0;
+    if (blocked && (rc = chol_plan_of(s, sc))) return rc;
+    // (blocks whose K changes every step, co-rotational ones, refactorise every step)
+    bool changing = false;
+    for (int q = 0; q < S.nsub; ++q) {
+        const SubDesc &u = s->sdesc[S.sub0 + q];
+        changing = changing || (u.tc && !u.cst);
+    }
+    const double *lam0 = P.lam0;
+    for (int step = 0; step < n_steps; ++step) {
+        const bool tc = s->gram[sc].njobs > 0 && (changing || !s->keep_factors || !s->grid_factored[sc]);
+        P.lam0 = step == 0 ? lam0 : nullptr;       // the learned start is the launch's first step's
+        P.tables = capturing || !s->grid_tables[sc];
+        P.tc_phase = tc ? 1 : 0;
+        P.tc_factor = tc && blocked ? 1 : 0;
+        // (between the steps of a call the kernels clear it for each other; an error stays)
+        if (step == 0) CK(cudaMemsetAsync(s->d_grid, 0, sizeof(GridScratch), st), "grid scratch");
+        if ((rc = coop_launch(s, setup, blocks, SUBADMM_THREADS, big ? need : 0, P, st))) return rc;
+        if (!capturing) s->grid_tables[sc] = 1;
+        if (tc) {
+            // the tensor-core map of the refactorised subsystems: the deferred FP32 factors (panel
+            // kernels and Schur updates) and their W, then the Gram kernel
+            if (blocked) {
+                CK(subadmm::chol_plan_run(s->chol[sc], st, &s->d_grid->err), "blocked factorisation launch");
+                P.tc_phase = 3;
+                P.tables = 0;
+                CK(cudaMemsetAsync(s->d_grid, 0, 2 * sizeof(unsigned), st), "grid barrier");
+                if ((rc = coop_launch(s, setup, blocks, SUBADMM_THREADS, 0, P, st))) return rc;
+            }
+            CK(subadmm::gram_plan_run(s->gram[sc], st, &s->d_grid->err), "Gram kernel launch");
+            if (s->keep_factors) s->grid_factored[sc] = 1;
+        }
+        P.tc_phase = 0;
+        // (a step that must agree on its end, or on a learned start, takes the barrier)
+        P.wave_tag = P.tol <= 0.0 && !P.lam0 ? plan.d_tag : nullptr;
+        if ((rc = coop_launch(s, iter, plan.blocks, SUBADMM_ITER, dyn, P, st))) return rc;
+    }
+    return SIM_OK;
+}
+
 int launch_grid_class(sim_t s, LaunchClass &c, StepParams P, cudaStream_t st, int split)
 {
     KernFn kf = grid_kernel_for(s->opt.precision == SIM_MIXED, split);
@@ -1383,7 +1694,19 @@ int launch_grid_class(sim_t s, LaunchClass &c, StepParams P, cudaStream_t st, in
     const int blocks = s->grid_blocks > 0 ? std::min(s->grid_blocks, resident)
                                           : std::max(1, resident / std::max(1, c.block_div));
     c.max_smem = 0;                 // reported: the largest stage buffers of the class's launches
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(st, &capturing), "capture status");
     for (size_t i = 0; i < c.scenes.size(); ++i) {
+        if (s->opt.stop != SIM_STOP_THETA) {
+            const int rc = iter_plan_of(s, c.scenes[i], iter_blocks(s, sms, c.block_div));
+            if (rc) return rc;
+            if (s->iter[c.scenes[i]].nwaves > 0) {
+                P.scene_ids = s->d_scene_ids + c.ids_off + (int)i;
+                const int rf = launch_grid_fused(s, c, P, st, c.scenes[i], capturing != cudaStreamCaptureStatusNone);
+                if (rf) return rf;
+                continue;
+            }
+        }
         // D rows staged in shared memory by bulk copies (the warp-per-row v-step only), two
         // stages per warp if that keeps the blocks per SM of the launch without them.  (The
         // kernel takes up to 4; on the FEM beam 3 and 4 measured slower than 2: the larger
@@ -1982,7 +2305,7 @@ int sim_probe_barrier(int device, int blocks, int expected, double limit_s, int 
     subadmm::DeviceGuard on_device(device);
     if (on_device.err != cudaSuccess) return SIM_ECUDA;
     int per_sm = 0, sms = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, subadmm::barrier_probe_kernel, 32, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, barrier_probe_kernel, 32, 0) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
         return SIM_ECUDA;
     if (blocks > per_sm * sms) return SIM_EINVAL;          // must all be resident
@@ -1994,7 +2317,7 @@ int sim_probe_barrier(int device, int blocks, int expected, double limit_s, int 
     unsigned ex = (unsigned)expected;
     unsigned long long lim = (unsigned long long)(limit_s * 1e9);
     void *args[] = {&count, &gen, &err, &ex, &lim, &passed};
-    cudaError_t e = cudaLaunchCooperativeKernel((const void *)subadmm::barrier_probe_kernel,
+    cudaError_t e = cudaLaunchCooperativeKernel((const void *)barrier_probe_kernel,
                                                 dim3(blocks), dim3(32), args, 0, nullptr);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     int host[2] = {0, 0};
