@@ -603,8 +603,8 @@ __device__ void map_item(const F *W, int n, int m, int mp, int ldd, int ldw, con
     }
 }
 
-// K_i = A_i + beta_i J_i^T J_i in FP32 for the blocks whose factorisation is left to the
-// blocked tensor-core factorisation (step flag 4, set before the barrier that precedes this),
+// K_i = A_i + beta_i J_i^T J_i (in the iteration type) for the blocks whose factorisation is
+// left to the banded or the blocked tensor-core factorisation (step flag 4, set before the barrier that precedes this),
 // a warp per row over every warp of the scene: the lower triangle from the first column of
 // the envelope's tile of the row's tile row on (zeros left of the envelope: that
 // factorisation reads whole tiles), then, for every row group whose span holds the row's
@@ -621,12 +621,14 @@ __device__ void deferred_fill(const StepParams &P, const SceneDesc &S, const Vie
         const int n = u.n;
         const SubEnv e = sub_env(P, u);
         const double *K = V.sdb + u.od_L, *J = V.sdb + u.od_J;
-        T *LT = V.stb + u.ot_L;
+        // (FP64: in place, A's band is there; what lies outside the envelope is never read)
+        constexpr bool COPY = sizeof(T) == 4;
+        T *LT = COPY ? V.stb + u.ot_L : reinterpret_cast<T *>(V.sdb + u.od_L);
         const T beta = (T)V.db[S.od_beta + i];
         for (int p = d.warp; p < n; p += d.nwarps) {
             const int ep = e.env[p], q0 = e.env[p & ~127] & ~127;
             T *Lp = LT + (size_t)p * n;
-            for (int q = q0 + lane; q <= p; q += 32) Lp[q] = q < ep ? (T)0 : (T)K[(size_t)p * n + q];
+            for (int q = q0 + lane; COPY && q <= p; q += 32) Lp[q] = q < ep ? (T)0 : (T)K[(size_t)p * n + q];
             __syncwarp();
             for (int g0 = 0; g0 < e.ngrp; g0 += 32) {
                 bool cov = false;
@@ -984,8 +986,8 @@ __device__ long long scene_setup(const StepParams &P, const SceneDesc &S, const 
             if (lane == 0) db[S.od_flag + i] = stiff ? 1.0 : 0.0;
         }
         bool ok;
-        const bool defer = MIXED && !stiff && P.tc_factor && P.tc_phase == 1 && u.tc;
-        if (stiff) {
+        const bool defer = (!MIXED || !stiff) && P.tc_factor && P.tc_phase == 1 && u.tc;
+        if (stiff && !defer) {
             add_jtj<double>(K, n, J, e, beta);
             ok = env_cholesky<double, false>(K, n, e, idg);
             if (ok) {
@@ -994,7 +996,7 @@ __device__ long long scene_setup(const StepParams &P, const SceneDesc &S, const 
                         LT[p * n + q] = (q == p) ? (T)idg[p] : (T)K[p * n + q];
             }
         } else if (defer) {
-            ok = true;                            // K in FP32 by deferred_fill, below
+            ok = true;                            // K by deferred_fill, below
         } else {
             for (int p = 0; p < n; ++p)
                 for (int q = e.env[p] + lane; q <= p; q += 32) LT[p * n + q] = (T)K[p * n + q];

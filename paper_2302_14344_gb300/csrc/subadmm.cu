@@ -20,6 +20,7 @@
 #include "device_guard.h"
 #include "gram.h"
 #include "chol.h"
+#include "band.h"
 
 using subadmm::KernFn;
 
@@ -136,6 +137,7 @@ struct sim_s {
     int tc_factor = 1;             // refactorised tc subsystems' FP32 factors by the blocked
                                    // Cholesky with tensor-core Schur updates
     std::vector<subadmm::CholPlan> chol;   // per scene: the blocked factorisation's panels
+    std::vector<subadmm::BandPlan> band;   // per scene: the banded factorisation of its tc subsystems
     std::vector<int> h_ipool;      // host copy of the integer pool (envelopes)
     std::vector<IterPlan> iter;            // per scene: grid scenes' iteration layout
     std::vector<char> grid_tables;         // per scene: its tables are in the workspace
@@ -298,6 +300,8 @@ void free_device(sim_t s)
     s->gram.clear();
     for (auto &c : s->chol) subadmm::chol_plan_free(c);
     s->chol.clear();
+    for (auto &b : s->band) subadmm::band_plan_free(b);
+    s->band.clear();
     s->grid_factored.clear();
     for (auto &p : s->iter) { cudaFree(p.d_lane); cudaFree(p.d_head); cudaFree(p.d_tag); }
     s->iter.clear();
@@ -330,6 +334,14 @@ int zeros(sim_t s, double **dst, size_t count, const char *what)
     e = cudaMemsetAsync(*dst, 0, std::max<size_t>(count, 1) * sizeof(double), s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, what);
     return SIM_OK;
+}
+
+// widest row of a subsystem's envelope
+int bandwidth(const std::vector<int> &ipool, const SubDesc &u)
+{
+    int w = 0;
+    for (int p = 0; p < u.n; ++p) w = std::max(w, p - ipool[u.env_off + p]);
+    return w;
 }
 
 int iter_blocks(const sim_t s, int sms, int div);
@@ -837,6 +849,10 @@ int finalize(sim_t s)
                 SubDesc &u = s->sdesc[S.sub0 + i];
                 u.tc = (s->tensor_cores && !s->pj && s->opt.precision == SIM_MIXED && u.n >= 128 &&
                         u.m >= 16) ? 1 : 0;
+                // (FP64: by the banded factorisation)
+                if (!s->pj && s->opt.precision == SIM_FP64 && s->opt.stop != SIM_STOP_THETA && u.n >= 128 &&
+                    u.m >= 16 && bandwidth(ipool, u) <= subadmm::kBandMax)
+                    u.tc = 1;
             }
             // everything in the workspace: the per-subsystem arrays, then the scene arrays
             S.sub_global = 1; S.hot_global = 1;
@@ -1372,7 +1388,7 @@ int gram_plan_of(sim_t s, int sc)
     float *stb = reinterpret_cast<float *>(tbase);
     for (int i = 0; i < S.nsub; ++i) {
         const SubDesc &u = s->sdesc[S.sub0 + i];
-        if (!u.tc) continue;
+        if (!u.tc || s->opt.precision != SIM_MIXED) continue;
         subadmm::GramJob J{};
         J.W = stb + u.ot_W;
         J.ldw = (u.m + 1 + 3) / 4 * 4;
@@ -1417,6 +1433,56 @@ int chol_plan_of(sim_t s, int sc)
     cudaError_t e = subadmm::chol_plan_build(C, mats, status, ST_NOTSPD);
     if (e == cudaErrorMemoryAllocation) return fail(s, SIM_ENOMEM, "blocked factorisation plan");
     CK(e, "blocked factorisation plan");
+    return SIM_OK;
+}
+
+// The banded factorisation plan of grid scene sc (its tc subsystems, if all of their envelopes are
+// narrow enough), built on first use.
+int band_plan_of(sim_t s, int sc)
+{
+    if ((int)s->band.size() < s->nscenes) {
+        s->band.resize(s->nscenes);
+        s->grid_factored.resize(s->nscenes, 0);
+    }
+    subadmm::BandPlan &B = s->band[sc];
+    if (B.device >= 0) return SIM_OK;
+    const SceneDesc &S = s->scenes[sc];
+    const bool fp64 = s->opt.precision == SIM_FP64;
+    double *sdb = reinterpret_cast<double *>(reinterpret_cast<char *>(s->d_work) + S.g_base);
+    char *stb = reinterpret_cast<char *>(s->d_work) + S.g_base + S.g_tbase;
+    const size_t ts = fp64 ? 8 : 4;
+    std::vector<subadmm::BandJob> jobs;
+    std::vector<std::vector<int>> jlo;
+    int bw = 0;
+    for (int i = 0; i < S.nsub; ++i) {
+        const SubDesc &u = s->sdesc[S.sub0 + i];
+        if (!u.tc) continue;
+        bw = std::max(bw, bandwidth(s->h_ipool, u));
+        subadmm::BandJob J{};
+        J.K = fp64 ? (void *)(sdb + u.od_L) : (void *)(stb + ts * u.ot_L);
+        J.LT = stb + ts * u.ot_L;
+        J.idg = sdb + u.od_id;
+        J.env = s->d_ipool + u.env_off;
+        J.lastr = J.env + u.n;
+        J.jlo = J.lastr + u.n;
+        J.jhi = J.jlo + u.m;
+        J.J = sdb + u.od_J;
+        J.b = sdb + u.od_b;
+        J.W = stb + ts * u.ot_W;
+        J.D = stb + ts * u.ot_D;
+        J.c = stb + ts * u.ot_c;
+        J.n = u.n; J.m = u.m; J.ldw = (u.m + 1 + 3) / 4 * 4; J.ldd = u.ldd; J.mpad = u.mpad;
+        J.pending = s->d_pending + S.sub0 + i;
+        J.subflag = u.cst ? s->d_subflag + S.sub0 + i : nullptr;
+        jobs.push_back(J);
+        const int *lo = s->h_ipool.data() + u.env_off + 2 * u.n;
+        jlo.emplace_back(lo, lo + u.m);
+    }
+    if (bw > subadmm::kBandMax) { jobs.clear(); jlo.clear(); }
+    int *status = reinterpret_cast<int *>(reinterpret_cast<char *>(s->d_grid) + offsetof(GridScratch, status));
+    cudaError_t e = subadmm::band_plan_build(B, jobs, jlo, bw, fp64, status, ST_NOTSPD);
+    if (e == cudaErrorMemoryAllocation) return fail(s, SIM_ENOMEM, "banded factorisation plan");
+    CK(e, "banded factorisation plan");
     return SIM_OK;
 }
 
@@ -1643,8 +1709,13 @@ int launch_grid_fused(sim_t s, LaunchClass &c, StepParams P, cudaStream_t st, in
     P.wave_smem = share;
     P.grid_big = big ? 1 : 0;
     int rc = gram_plan_of(s, sc);
-    if (rc) return rc;
-    const bool blocked = s->tc_factor && s->gram[sc].njobs > 0;
+    if (rc || (rc = band_plan_of(s, sc))) return rc;
+    // refactorised large blocks: the banded factorisation where all envelopes are narrow (always in
+    // FP64), else (FP32) the blocked one on the tensor cores, which serves dense blocks; with
+    // sim_tc_factor(0) the mixed form's factors stay in the setup, a warp per block
+    const bool factor = !mixed || s->tc_factor;
+    const bool banded = factor && s->band[sc].njobs > 0;
+    const bool blocked = factor && !banded && s->gram[sc].njobs > 0;
     if (blocked && (rc = chol_plan_of(s, sc))) return rc;
     // (blocks whose K changes every step, co-rotational ones, refactorise every step)
     bool changing = false;
@@ -1654,26 +1725,28 @@ int launch_grid_fused(sim_t s, LaunchClass &c, StepParams P, cudaStream_t st, in
     }
     const double *lam0 = P.lam0;
     for (int step = 0; step < n_steps; ++step) {
-        const bool tc = s->gram[sc].njobs > 0 && (changing || !s->keep_factors || !s->grid_factored[sc]);
+        const bool tc = (s->gram[sc].njobs > 0 || banded) && (changing || !s->keep_factors || !s->grid_factored[sc]);
         P.lam0 = step == 0 ? lam0 : nullptr;       // the learned start is the launch's first step's
         P.tables = capturing || !s->grid_tables[sc];
         P.tc_phase = tc ? 1 : 0;
-        P.tc_factor = tc && blocked ? 1 : 0;
+        P.tc_factor = tc && (banded || blocked) ? 1 : 0;
         // (between the steps of a call the kernels clear it for each other; an error stays)
         if (step == 0) CK(cudaMemsetAsync(s->d_grid, 0, sizeof(GridScratch), st), "grid scratch");
         if ((rc = coop_launch(s, setup, blocks, SUBADMM_THREADS, big ? need : 0, P, st))) return rc;
         if (!capturing) s->grid_tables[sc] = 1;
         if (tc) {
-            // the tensor-core map of the refactorised subsystems: the deferred FP32 factors (panel
-            // kernels and Schur updates) and their W, then the Gram kernel
+            if (banded) CK(subadmm::band_plan_run(s->band[sc], st), "banded factorisation launch");
             if (blocked) {
+                // panel kernels and Schur updates, then W of those subsystems
                 CK(subadmm::chol_plan_run(s->chol[sc], st, &s->d_grid->err), "blocked factorisation launch");
                 P.tc_phase = 3;
                 P.tables = 0;
                 CK(cudaMemsetAsync(s->d_grid, 0, 2 * sizeof(unsigned), st), "grid barrier");
                 if ((rc = coop_launch(s, setup, blocks, SUBADMM_THREADS, 0, P, st))) return rc;
             }
-            CK(subadmm::gram_plan_run(s->gram[sc], st, &s->d_grid->err), "Gram kernel launch");
+            // the mixed form's D and c: the tensor-core Gram kernel
+            if (s->gram[sc].njobs > 0)
+                CK(subadmm::gram_plan_run(s->gram[sc], st, &s->d_grid->err), "Gram kernel launch");
             if (s->keep_factors) s->grid_factored[sc] = 1;
         }
         P.tc_phase = 0;

@@ -69,3 +69,23 @@ def test_stop_at_the_tolerance():
         r, q = sim.residuals(k), o.residuals()
         assert r["converged"] and r["iters"] == q["iters"]
         assert _rel(sim.scene_vhat(k), o.vhat_all()) < 1e-9
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("ny,nz,planes,slabs", [(7, 7, 4, 1), (8, 9, 6, 2), (10, 10, 8, 3)])
+def test_refactorised_bands(precision, ny, nz, planes, slabs):
+    """Co-rotational slabs (n = 588 .. 1200, ragged against the panels of 16 and 32 columns), refactorised
+    every step by the banded factorisation, against the oracle over two steps."""
+    p = sg.fem_beam(0, ny=ny, nz=nz, planes=planes, slabs=slabs, length=0.004 * planes, corotational=True,
+                    with_gripper=False, tol_primal=-1, max_iters=15)
+    for sim, k, o in _run(p, steps=1, calls=2, precision=precision):
+        assert _rel(sim.scene_vhat(k), o.vhat_all()) < (1e-4 if precision else 1e-9)
+        assert _rel(sim.scene_nodes(k), o.nodes_all()) < (1e-5 if precision else 1e-9)
+
+
+def test_wide_envelopes_take_the_tensor_core_factorisation():
+    """Dense blocks (envelopes wider than the banded factorisation takes) in the mixed form, every
+    step refactorised: the blocked factorisation on the tensor cores, against the oracle."""
+    p = sg.generic(9, n_scenes=1, n_sub=3, n_range=(400, 420), extra=12, tol_primal=-1, max_iters=20, warm="prev")
+    for sim, k, o in _run(p, steps=1, calls=2, precision=1):
+        assert _rel(sim.scene_vhat(k), o.vhat_all()) < 1e-4
