@@ -17,6 +17,7 @@
 #define SUBADMM_MAXN 2048       // largest subsystem DOF
 #define SUBADMM_MAXM 2048       // largest side-row count of one subsystem
 #define SUBADMM_ITER 512        // threads of the grid's iteration kernel (one block per SM)
+#define SUBADMM_OWN 3           // side-rows a thread may own in the block kernel's generic iteration
 #define SUBADMM_BIG 96          // grid kernel: DOF from which a block solves a subsystem
 #define SUBADMM_PARAMS 23       // doubles of a rigid-model constraint's parameters
 #define SUBADMM_BODY 17         // doubles of a body record
@@ -92,6 +93,7 @@ struct SubDesc {
                            // X0 (n), K values (linear)
     int csr_off;           // linear: ipool offset of the K row pointers (n+1), then columns
     int env_off;           // ipool offset of the profile of K_i: env (n), lastr (n), jlo (m), jhi (m)
+    int bw;                // widest row of the envelope: largest p - env[p]
     int grp_off, ngrp;     // ipool offset of the row groups of J_ci: maximal runs of consecutive
                            // rows with one column span, as ngrp + 1 first rows (the last = m)
     int cst;               // 1 if K_i is the same at every step (its factor may be kept)
@@ -101,6 +103,8 @@ struct SubDesc {
     int ot_L, ot_W;        // T region: L (n x n, 1/L_pp on the diagonal); W = L^-1 [J^T b]
                            // (n x (m + 1), column-major: W[p (m + 1) + t], column m = g)
     int ot_s;              // T region: solve vector of the mixed recovery (n)
+    int ot_Dres;           // scene T region (shared memory): copy of D for the iterations of a block
+                           // scene whose D lives in the workspace (-1: none)
     int ot_D, ot_c;        // iteration region: D (m rows of mpad, ldd apart), c (m)
     int v_off;             // global offset of v-hat
     int ne, tet_off, ke_off;   // co-rotational linear block: elements, ipool offset of their
@@ -229,6 +233,13 @@ SUBADMM_HD inline size_t block_solve_groups(int ngrp) { return (size_t)(3 * ngrp
 SUBADMM_HD inline size_t block_solve_bytes(int n, int ngrp)
 {
     return block_solve_groups(ngrp) + 8 * ((size_t)(n + 1) / 2 * 2 + 2 * kPanel * kTileLd) + 4 * (size_t)n;
+}
+
+// D chunks (16-byte vectors) a lane keeps in registers in the block kernel's register-cached
+// iteration, by lanes per side-row: rows of up to 32 side-rows in FP32 and 24, 32 or 48 in FP64
+SUBADMM_HD constexpr int cached_chunks(int tsize, int split)
+{
+    return tsize == 4 ? (split == 1 ? 8 : 4) : split == 1 ? 12 : split == 2 ? 8 : 6;
 }
 
 // Vectors (16 bytes) per lane of a wide row in a wave of shape B: 256 side-rows of a subsystem

@@ -37,6 +37,7 @@
 #include "layout.h"
 #include "rigid_model.cuh"
 #include "block_solve.cuh"
+#include "band_warp.cuh"
 
 namespace subadmm {
 
@@ -90,15 +91,18 @@ __device__ __forceinline__ unsigned tol_bits(float, double tol) { return __float
 __device__ __forceinline__ unsigned long long tol_bits(double, double tol) { return rbits(tol); }
 __device__ __forceinline__ unsigned inf_bits(float) { return 0x7f800000u; }
 __device__ __forceinline__ unsigned long long inf_bits(double) { return 0x7ff0000000000000ull; }
-// D chunks (16-byte vectors) a lane keeps in registers in the cached iteration
-template <typename T> struct CachedChunks;
-template <> struct CachedChunks<float> { static constexpr int value = 4; };
-template <> struct CachedChunks<double> { static constexpr int value = 6; };
 template <typename T> struct VecZero;
 template <> struct VecZero<float> { __device__ static float4 get() { return make_float4(0.f, 0.f, 0.f, 0.f); } };
 template <> struct VecZero<double> { __device__ static double2 get() { return make_double2(0.0, 0.0); } };
+// a > 0 (a NaN counts as positive), on the integer pipe
+__device__ __forceinline__ bool above0(float a) { return __float_as_int(a) > 0; }
+__device__ __forceinline__ bool above0(double a) { return __double_as_longlong(a) > 0; }
 __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
+
+}  // namespace subadmm
+#include "own_iter.cuh"
+namespace subadmm {
 
 // Sum (a) and maxima (b, c) of three per-thread doubles over the block.
 __device__ __forceinline__ void block_reduce3(double (*red)[SUBADMM_MAXWARPS], double &a,
@@ -166,6 +170,7 @@ struct View {
     T *htb;              // per-subsystem iteration arrays (D, c): shared memory unless the
                          // scene cannot hold even those
     int *row, *sub, *drow, *coff, *wbase, *mlen;   // per side-row tables
+    int *meta;           // other side's side-row of the row + 1 | type << 16 | row of its contact << 18
     Item *item;
     int *list;
 };
@@ -192,9 +197,19 @@ __device__ View<T> scene_view(const StepParams &P, const SceneDesc &S, unsigned 
     V.coff = ib + 3 * S.nsr;
     V.wbase = ib + 4 * S.nsr;
     V.mlen = ib + 5 * S.nsr;
-    V.item = reinterpret_cast<Item *>(ib + 6 * S.nsr);
-    V.list = ib + 6 * S.nsr + 4 * S.nitem;
+    V.meta = ib + 6 * S.nsr;
+    V.item = reinterpret_cast<Item *>(ib + (7 * S.nsr + 3) / 4 * 4);
+    V.list = ib + (7 * S.nsr + 3) / 4 * 4 + 4 * S.nitem;
     return V;
+}
+
+// D row of a side-row: in the iteration arrays, or (complemented offset) the scene's copy in
+// shared memory
+template <typename T>
+__device__ __forceinline__ const typename VecOf<T>::V *d_row(const View<T> &V, int t)
+{
+    const int o = V.drow[t];
+    return reinterpret_cast<const typename VecOf<T>::V *>(o < 0 ? V.tb + ~o : V.htb + o);
 }
 
 // Work distribution of one scene's step: the threads of a block (block kernel: one block
@@ -282,6 +297,7 @@ __device__ void scene_tables(const StepParams &P, const SceneDesc &S, const View
 {
     for (int t = d.tid; t < S.nsr; t += d.nthreads) {
         V.row[t] = 0; V.sub[t] = 0; V.drow[t] = 0; V.coff[t] = 0; V.wbase[t] = 0; V.mlen[t] = 0;
+        V.meta[t] = 0;
     }
     d.sync();
     for (int j = d.tid; j < S.ncon; j += d.nthreads) {
@@ -293,10 +309,11 @@ __device__ void scene_tables(const StepParams &P, const SceneDesc &S, const View
                 const int lr = t - u.sr0;
                 V.row[t] = c.row0 + r;
                 V.sub[t] = c.sub[s];
-                V.drow[t] = u.ot_D + lr * u.ldd;
+                V.drow[t] = u.ot_Dres >= 0 ? ~(u.ot_Dres + lr * u.ldd) : u.ot_D + lr * u.ldd;
                 V.coff[t] = u.ot_c + lr;
                 V.wbase[t] = u.sr0;
                 V.mlen[t] = u.m;
+                V.meta[t] = (c.ns == 2 ? c.sr[s ^ 1] + r + 1 : 0) | c.type << 16 | (c.type == TYPE_CONTACT ? r << 18 : 0);
             }
         }
     }
@@ -349,6 +366,58 @@ __device__ __forceinline__ SubEnv sub_env(const StepParams &P, const SubDesc &u)
     return e;
 }
 
+// The row groups of a subsystem for one warp, 32 at a time in its lanes' registers: f(r0, r1, lo, w)
+// for every group in order (rows r0 .. r1 - 1, columns lo .. lo + w - 1).  The setup's loops over
+// groups and rows are chains of short passes; with their tables read as they went, each pass
+// waited for two more trips to L2 (the tables of a scene whose arrays fill shared memory do not
+// stay in the L1 that is left).
+template <typename Fn>
+__device__ __forceinline__ void for_groups(const SubEnv &e, Fn f)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    for (int g0 = 0; g0 < e.ngrp; g0 += 32) {
+        const int g = min(g0 + lane, e.ngrp - 1);
+        const int r0 = e.grp[g], r1 = e.grp[g + 1], lo = e.jlo[r0], w = e.jhi[r0] - lo;
+        const int cnt = min(32, e.ngrp - g0);
+        for (int q = 0; q < cnt; ++q)
+            f(__shfl_sync(FULL, r0, q), __shfl_sync(FULL, r1, q), __shfl_sync(FULL, lo, q), __shfl_sync(FULL, w, q));
+    }
+}
+
+// Rows p of a band, 4 at a time: entries lo(p) .. hi(p) of src, converted by conv(p, q, value), into
+// dst (row length n); every load of a pass before its stores
+template <typename D, typename S, typename Conv>
+__device__ __forceinline__ void copy_band(D *dst, const S *src, int n, const int *lo, Conv conv)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    for (int b = 0; b < n; b += 32) {
+        const int el = lo[min(b + lane, n - 1)];
+        for (int h = 0; h < 32 && b + h < n; h += 4) {
+            int e[4], len = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                e[i] = __shfl_sync(FULL, el, h + i);
+                if (b + h + i < n) len = max(len, b + h + i - e[i] + 1);
+            }
+            for (int c = lane; c < (len + 31) / 32 * 32; c += 32) {
+                S v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int p = b + h + i, q = e[i] + c;
+                    v[i] = p < n && q <= p ? src[(size_t)p * n + q] : (S)0;
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int p = b + h + i, q = e[i] + c;
+                    if (p < n && q <= p) dst[(size_t)p * n + q] = conv(p, q, v[i]);
+                }
+            }
+        }
+    }
+}
+
 // A constant K_i whose factor from an earlier step is still held: in the workspace (it
 // outlives the launch) or in shared memory from an earlier step of this launch.  With
 // keep_factors 0 every step refactors (the same matrix; results agree to rounding).  A
@@ -370,19 +439,18 @@ template <typename F>
 __device__ void add_jtj(F *K, int n, const double *J, const SubEnv &e, F beta)
 {
     const int lane = threadIdx.x & 31;
-    for (int g = 0; g < e.ngrp; ++g) {
-        const int r0 = e.grp[g], r1 = e.grp[g + 1];
-        const int lo = e.jlo[r0], w = e.jhi[r0] - lo;
+    for_groups(e, [&](int r0, int r1, int lo, int w) {
         const double *J0 = J + (size_t)r0 * n + lo;
         for (int k = lane; k < w * (w + 1) / 2; k += 32) {
             int a, b;
             tri_index(k, a, b);
+            const F old = K[(lo + a) * n + lo + b];
             F acc = (F)0;
             for (int t = 0; t < r1 - r0; ++t) acc += (F)J0[(size_t)t * n + a] * (F)J0[(size_t)t * n + b];
-            K[(lo + a) * n + lo + b] += beta * acc;
+            K[(lo + a) * n + lo + b] = old + beta * acc;
         }
         __syncwarp();
-    }
+    });
 }
 
 // Right-looking Cholesky inside the envelope, in place on the lower triangle of K (one
@@ -392,6 +460,67 @@ __device__ void add_jtj(F *K, int n, const double *J, const SubEnv &e, F beta)
 // instruction occupies its pipe however few lanes are active).  Every entry receives the
 // same updates in the same order (k ascending).  INV_DIAG: the diagonal ends as 1/L_kk
 // (the T factor); otherwise as L_kk with 1/L_kk in idg.  False on a non-positive pivot.
+// Columns that reach at most 31 rows (narrow bands: rigid chains, spring blocks): the scaled column
+// is in the lanes' registers (its entries go round by shuffles), the triangle's indices are
+// worked out once, and every entry of a pass is loaded before any is stored (the compiler cannot
+// move a load of K above a store to K: a 23-wide column cost nine round trips to L2, some 6k
+// cycles, where it now costs one).
+template <typename F, bool INV_DIAG>
+__device__ bool narrow_cholesky(F *K, int n, const SubEnv &e, double *idg)
+{
+    constexpr int PASS = 5;                        // 32-entry slots per pass: 3 passes cover w = 30
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    unsigned char ia[3 * PASS + 1], ib[3 * PASS + 1];
+#pragma unroll
+    for (int s = 0; s < 3 * PASS + 1; ++s) {
+        int a, b;
+        tri_index(lane + 32 * s, a, b);
+        ia[s] = (unsigned char)a;
+        ib[s] = (unsigned char)b;
+    }
+    for (int k = 0; k < n; ++k) {
+        const int w = e.lastr[k] - k, tri = w * (w + 1) / 2;
+        const F d = K[(size_t)k * n + k];
+        F l = lane < w ? K[(size_t)(k + 1 + lane) * n + k] : (F)0;
+        if (!(d > (F)0) || !isfinite(d)) return false;
+        F *const T0 = K + (size_t)(k + 1) * n + k + 1;
+        F c[PASS];
+#pragma unroll
+        for (int s = 0; s < PASS; ++s) c[s] = lane + 32 * s < tri ? T0[(size_t)ia[s] * n + ib[s]] : (F)0;
+        const F ilkk = rsq(d);
+        l *= ilkk;
+        __syncwarp();                              // every lane has read the pivot and the column
+        if (lane < w) K[(size_t)(k + 1 + lane) * n + k] = l;
+        if (lane == 0) {
+            if (INV_DIAG) {
+                K[(size_t)k * n + k] = ilkk;
+            } else {
+                K[(size_t)k * n + k] = d * ilkk;
+                idg[k] = (double)ilkk;
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < 3 * PASS + 1; p += PASS) {
+            if (32 * p >= tri) break;
+            if (p > 0)
+#pragma unroll
+                for (int s = 0; s < PASS; ++s)
+                    if (p + s < 3 * PASS + 1)
+                        c[s] = lane + 32 * (p + s) < tri ? T0[(size_t)ia[p + s < 3 * PASS + 1 ? p + s : 0] * n + ib[p + s < 3 * PASS + 1 ? p + s : 0]] : (F)0;
+#pragma unroll
+            for (int s = 0; s < PASS; ++s) {
+                const int q = p + s < 3 * PASS + 1 ? p + s : 0;
+                if (p + s >= 3 * PASS + 1 || 32 * (p + s) >= tri) continue;
+                const F la = __shfl_sync(FULL, l, ia[q]), lb = __shfl_sync(FULL, l, ib[q]);
+                if (lane + 32 * (p + s) < tri) T0[(size_t)ia[q] * n + ib[q]] = c[s] - la * lb;
+            }
+        }
+        __syncwarp();
+    }
+    return true;
+}
+
 template <typename F, bool INV_DIAG>
 __device__ bool env_cholesky(F *K, int n, const SubEnv &e, double *idg)
 {
@@ -539,6 +668,17 @@ __device__ void env_forward_vec(const F *LT, F *y, int n, int ldy, const int *la
     }
 }
 
+__device__ __forceinline__ void load_quad(const float *p, float *v)
+{
+    const float4 a = *reinterpret_cast<const float4 *>(p);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+}
+__device__ __forceinline__ void load_quad(const double *p, double *v)
+{
+    const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+
 // One work item of the map D = W^T W, c = W^T g of a subsystem (W = L^-1 [J^T b], column m
 // is g; W column t is zero above row jlo[t]; D rows ldd apart, zero-padded from m to mp), for
 // items spread over many threads: item k < nb (nb + 1) / 2 is the 4 x 4 block k of D's lower
@@ -565,11 +705,12 @@ __device__ void map_item(const F *W, int n, int m, int mp, int ldd, int ldw, con
         for (int a = 0; a < 4; ++a)
 #pragma unroll
             for (int b = 0; b < 4; ++b) acc[a][b] = (F)0;
+#pragma unroll 4
         for (int p = max(pr, ps); p < n; ++p) {
-            const F *Wp = W + (size_t)p * ldw;
+            const F *Wp = W + (size_t)p * ldw;             // (16-byte aligned, as r0 and s0 are)
             F wr[4], ws[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) { wr[q] = Wp[r0 + q]; ws[q] = Wp[s0 + q]; }
+            load_quad(Wp + r0, wr);
+            load_quad(Wp + s0, ws);
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -691,9 +832,10 @@ __device__ void w_chunks(const StepParams &P, const SceneDesc &S, const View<T> 
             if (flag != want) continue;
             const SubDesc &u = P.subs[S.sub0 + i];
             const int ldw = (u.m + 1 + 3) / 4 * 4;
+            const int c0 = 32 * (w - __ldg(wpre + pos));
+            const bool whole = (P.tc_phase == 1 || P.tc_phase == 3) && u.tc;
             solve_w_chunk<T>(stb + u.ot_L, stb + u.ot_W, sdb + u.od_J, sdb + u.od_b, u.n, u.m,
-                             ldw, 32 * (w - __ldg(wpre + pos)), sub_env(P, u),
-                             (P.tc_phase == 1 || P.tc_phase == 3) && u.tc);
+                             ldw, c0, sub_env(P, u), whole);
         }
     }
 }
@@ -715,11 +857,10 @@ __device__ long long scene_setup(const StepParams &P, const SceneDesc &S, const 
         double *J = sdb + u.od_J, *K = sdb + u.od_L;
         // J's rows are read only inside their column spans (model rows are written there,
         // explicit rows whole): zero the spans
-        for (int g = 0; g < e.ngrp; ++g) {
-            const int r0 = e.grp[g], r1 = e.grp[g + 1], lo = e.jlo[r0], w = e.jhi[r0] - lo;
+        for_groups(e, [&](int r0, int r1, int lo, int w) {
             for (int k = lane; k < (r1 - r0) * w; k += 32)
                 J[(size_t)(r0 + k / w) * u.n + lo + k % w] = 0.0;
-        }
+        });
         if (u.kind == KIND_GENERIC) {
             const double *A = P.pool + u.gen_off;
             for (int q = lane; q < u.n * u.n; q += 32) K[q] = A[q];
@@ -728,8 +869,14 @@ __device__ long long scene_setup(const StepParams &P, const SceneDesc &S, const 
         }
         if (!keep) {
             // the band [env[p], lastr[p]] of every row holds A (both triangles)
-            for (int p = 0; p < u.n; ++p)
-                for (int q = e.env[p] + lane; q <= e.lastr[p]; q += 32) K[p * u.n + q] = 0.0;
+            for (int b = 0; b < u.n; b += 32) {
+                const int pl = min(b + lane, u.n - 1), lo = e.env[pl], hi = e.lastr[pl];
+                for (int h = 0; h < 32 && b + h < u.n; ++h) {
+                    const int q1 = __shfl_sync(0xffffffffu, hi, h);
+                    for (int q = __shfl_sync(0xffffffffu, lo, h) + lane; q <= q1; q += 32)
+                        K[(size_t)(b + h) * u.n + q] = 0.0;
+                }
+            }
         }
         if (u.kind == KIND_LINEAR) {
             // A = (2/h) M + (h/2) K_el (K_el sparse, scattered into the band);
@@ -921,26 +1068,24 @@ __device__ long long scene_setup(const StepParams &P, const SceneDesc &S, const 
         if (!MIXED) {
             double trA = 0.0, trJ = 0.0;
             for (int q = lane; q < n; q += 32) trA += K[q * n + q];
-            for (int g = 0; g < e.ngrp; ++g) {            // J's rows inside their spans
-                const int r0 = e.grp[g], r1 = e.grp[g + 1], lo = e.jlo[r0], w = e.jhi[r0] - lo;
+            for_groups(e, [&](int r0, int r1, int lo, int w) {      // J's rows inside their spans
                 for (int k = lane; k < (r1 - r0) * w; k += 32) {
                     const double x = J[(size_t)(r0 + k / w) * n + lo + k % w];
                     trJ += x * x;
                 }
-            }
+            });
             trA = warp_sum(trA);
             trJ = warp_sum(trJ);
             beta = P.beta_fixed ? P.rho : (trJ > 0.0 ? trA / trJ : 1.0);
         } else {
             T trA = (T)0, trJ = (T)0;
             for (int q = lane; q < n; q += 32) trA += (T)K[q * n + q];
-            for (int g = 0; g < e.ngrp; ++g) {
-                const int r0 = e.grp[g], r1 = e.grp[g + 1], lo = e.jlo[r0], w = e.jhi[r0] - lo;
+            for_groups(e, [&](int r0, int r1, int lo, int w) {
                 for (int k = lane; k < (r1 - r0) * w; k += 32) {
                     const T jq = (T)J[(size_t)(r0 + k / w) * n + lo + k % w];
                     trJ += jq * jq;
                 }
-            }
+            });
 #pragma unroll
             for (int o = 16; o; o >>= 1) {
                 trA += __shfl_xor_sync(0xffffffffu, trA, o);
@@ -961,16 +1106,17 @@ __device__ long long scene_setup(const StepParams &P, const SceneDesc &S, const 
             // below; a stiff or high-mass-ratio block (spread > 1e3) is factorised in FP64
             const T bt = (T)beta;
             T dmax = (T)0, dmin = (T)3.0e38;
-            for (int p = lane; p < n; p += 32) {
+            for (int b = 0; b < n; b += 32) {
+                const int p = b + lane;
                 T cs = (T)0;                       // rows whose span holds column p, in order
-                for (int g = 0; g < e.ngrp; ++g) {
-                    const int r0 = e.grp[g];
-                    if (p < e.jlo[r0] || p >= e.jhi[r0]) continue;
-                    for (int r = r0; r < e.grp[g + 1]; ++r) {
-                        const T jr = (T)J[r * n + p];
+                for_groups(e, [&](int r0, int r1, int lo, int w) {
+                    if (p < lo || p >= lo + w) return;
+                    for (int r = r0; r < r1; ++r) {
+                        const T jr = (T)J[(size_t)r * n + p];
                         cs += jr * jr;
                     }
-                }
+                });
+                if (p >= n) continue;
                 const T dk = (T)K[p * n + p] + bt * cs;
                 dmax = dk > dmax ? dk : dmax;
                 dmin = dk < dmin ? dk : dmin;
@@ -989,20 +1135,19 @@ __device__ long long scene_setup(const StepParams &P, const SceneDesc &S, const 
         const bool defer = (!MIXED || !stiff) && P.tc_factor && P.tc_phase == 1 && u.tc;
         if (stiff && !defer) {
             add_jtj<double>(K, n, J, e, beta);
-            ok = env_cholesky<double, false>(K, n, e, idg);
+            ok = u.bw <= kNarrowBand ? narrow_cholesky<double, false>(K, n, e, idg)
+                                     : env_cholesky<double, false>(K, n, e, idg);
             if (ok) {
-                for (int p = 0; p < n; ++p)
-                    for (int q = e.env[p] + lane; q <= p; q += 32)
-                        LT[p * n + q] = (q == p) ? (T)idg[p] : (T)K[p * n + q];
+                copy_band(LT, K, n, e.env, [&](int p, int q, double v) { return q == p ? (T)idg[p] : (T)v; });
             }
         } else if (defer) {
             ok = true;                            // K by deferred_fill, below
         } else {
-            for (int p = 0; p < n; ++p)
-                for (int q = e.env[p] + lane; q <= p; q += 32) LT[p * n + q] = (T)K[p * n + q];
+            copy_band(LT, K, n, e.env, [](int, int, double v) { return (T)v; });
             __syncwarp();
             add_jtj<T>(LT, n, J, e, (T)beta);
-            ok = env_cholesky<T, true>(LT, n, e, nullptr);
+            ok = u.bw <= kNarrowBand ? narrow_cholesky<T, true>(LT, n, e, nullptr)
+                                     : env_cholesky<T, true>(LT, n, e, nullptr);
         }
         if (u.cst && lane == 0) P.subflag[gsub] = ok ? (1 | (stiff ? 2 : 0)) : 0;
         __syncwarp();
@@ -1116,23 +1261,29 @@ __device__ __forceinline__ void add_jt(double *out, const double *J, int n, cons
                                        const W *w)
 {
     const int lane = threadIdx.x & 31;
-    for (int g = 0; g < e.ngrp; ++g) {
-        const int r0 = e.grp[g], r1 = e.grp[g + 1];
-        for (int p = e.jlo[r0] + lane; p < e.jhi[r0]; p += 32) {
+    for_groups(e, [&](int r0, int r1, int lo, int sw) {
+        for (int p = lo + lane; p < lo + sw; p += 32) {
+            const double old = out[p];
             double acc = 0.0;
             for (int r = r0; r < r1; ++r) acc += J[(size_t)r * n + p] * (double)w[r];
-            out[p] += acc;
+            out[p] = old + acc;
         }
         __syncwarp();
-    }
+    });
 }
 
 // Triangular solves with the T factor (1/L_pp on its diagonal), in place on s (warp),
 // inside the envelope.
 template <typename T>
-__device__ __forceinline__ void warp_chol_solve(const T *LT, T *s, int n, const SubEnv &e)
+__device__ __forceinline__ void warp_chol_solve(const T *LT, T *s, int n, const SubEnv &e, int bw)
 {
     const int lane = threadIdx.x & 31;
+    if (bw <= kNarrowBand) {
+        auto inv = [LT, n](int r) { return LT[(size_t)r * n + r]; };
+        warp_band_forward<T>(LT, n, e.env, s, inv);
+        warp_band_backward<T>(LT, n, e.env, s, inv);
+        return;
+    }
     for (int p = 0; p < n; ++p) {              // L y = s (column-oriented)
         const T yp = s[p] * LT[p * n + p];
         __syncwarp();
@@ -1280,6 +1431,12 @@ __device__ void recover_v(const StepParams &P, const SceneDesc &S, const View<T>
             for (int p = lane; p < n; p += 32) v[p] = b[p];
             __syncwarp();
             add_jt(v, J, n, e, wi);
+            if (u.bw <= kNarrowBand) {
+                auto inv = [idg](int r) { return idg[r]; };
+                warp_band_forward<double>(Lf, n, e.env, v, inv);
+                warp_band_backward<double>(Lf, n, e.env, v, inv);
+                continue;
+            }
             for (int p = 0; p < n; ++p) {          // L y = rhs (column-oriented)
                 const double yp = v[p] * idg[p];
                 __syncwarp();
@@ -1306,7 +1463,7 @@ __device__ void recover_v(const StepParams &P, const SceneDesc &S, const View<T>
         add_jt(rhs, J, n, e, wi);
         for (int p = lane; p < n; p += 32) s[p] = (T)rhs[p];
         __syncwarp();
-        warp_chol_solve<T>(LT, s, n, e);
+        warp_chol_solve<T>(LT, s, n, e, u.bw);
         for (int p = lane; p < n; p += 32) v[p] = (double)s[p];
         __syncwarp();
         // one refinement step: r = rhs - A v - beta J^T (J v); v += K^-1 r.  Row p of A lies
@@ -1327,7 +1484,7 @@ __device__ void recover_v(const StepParams &P, const SceneDesc &S, const View<T>
             s[p] = (T)acc;
         }
         __syncwarp();
-        warp_chol_solve<T>(LT, s, n, e);
+        warp_chol_solve<T>(LT, s, n, e, u.bw);
         for (int p = lane; p < n; p += 32) v[p] += (double)s[p];
         __syncwarp();
     }
@@ -1553,60 +1710,6 @@ struct RegItem {
         return mloc;
     }
 
-    // lambda of the item (Sec. III-C) from the y of its side-rows, slot s * rows + r.  In
-    // FP32 one instruction stream serves every type (a warp holds items of several types):
-    // the first row is -(a q + e) s with (a, s) = (alpha, k) for soft rows and
-    // (1, 1 / sum 1/beta) otherwise, clamped at 0 for hard and contact rows; contact rows 1, 2
-    // are then scaled into the friction cone.  In FP64, where every instruction is costly,
-    // each type runs only its own formula.
-    __device__ __forceinline__ void lambda_of(const T *ys, T *lv) const
-    {
-        const bool two = t1 >= 0, con = nr == 3;
-        if constexpr (sizeof(T) == 4) {
-            const T yb0 = two ? (con ? ys[3] : ys[1]) : (T)0;
-            const T q0 = ys[0] * ib0 + yb0 * ib1;
-            const T a0 = type == TYPE_SOFT ? al : (T)1;
-            const T s0 = type == TYPE_SOFT ? kf : is;
-            T l0 = -(q0 * a0 + e0) * s0;
-            if (type == TYPE_HARD || con) l0 = l0 > (T)0 ? l0 : (T)0;
-            const T yb1 = two ? ys[4] : (T)0, yb2 = two ? ys[5] : (T)0;
-            const T l1 = -(ys[1] * ib0 + yb1 * ib1 + e1) * is;
-            const T l2 = -(ys[2] * ib0 + yb2 * ib1 + e2) * is;
-            const T t2 = l1 * l1 + l2 * l2;
-            const T lim = mu * l0;
-            const T f = t2 > lim * lim ? lim * rsq(t2) : (T)1;
-            const bool on = valid && con && l0 > (T)0;
-            lv[0] = valid ? l0 : (T)0;
-            lv[1] = on ? l1 * f : (T)0;
-            lv[2] = on ? l2 * f : (T)0;
-        } else {
-            lv[0] = lv[1] = lv[2] = (T)0;
-            if (!valid) return;
-            if (con) {
-                const T yb0 = two ? ys[3] : (T)0, yb1 = two ? ys[4] : (T)0, yb2 = two ? ys[5] : (T)0;
-                const T ln = -(ys[0] * ib0 + yb0 * ib1 + e0) * is;
-                if (ln > (T)0) {
-                    const T l1 = -(ys[1] * ib0 + yb1 * ib1 + e1) * is;
-                    const T l2 = -(ys[2] * ib0 + yb2 * ib1 + e2) * is;
-                    const T t2 = l1 * l1 + l2 * l2;
-                    const T lim = mu * ln;
-                    lv[0] = ln;
-                    if (t2 > lim * lim) { const T f = lim * rsq(t2); lv[1] = l1 * f; lv[2] = l2 * f; }
-                    else { lv[1] = l1; lv[2] = l2; }
-                }
-            } else {
-                const T q = ys[0] * ib0 + (two ? ys[1] : (T)0) * ib1;
-                T l;
-                if (type == TYPE_SOFT) l = -(e0 + al * q) * kf;
-                else {
-                    l = -(q + e0) * is;
-                    if (type == TYPE_HARD) l = l > (T)0 ? l : (T)0;
-                }
-                lv[0] = l;
-            }
-        }
-    }
-
     // write the z (and the previous z) held in registers back to the scene arrays
     __device__ __forceinline__ void publish(T *Z, T *ZO) const
     {
@@ -1639,6 +1742,7 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
     __shared__ U ured[2][NW];
     __shared__ T tred[2][NW];
     __shared__ int s_status;
+    __shared__ SceneDesc s_scene;          // (own_iterate)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr bool MIXED = sizeof(T) == 4;
 
@@ -1646,6 +1750,7 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
         const int sc = P.scene_ids[k];
         const SceneDesc S = P.scenes[sc];
         const View<T> V = scene_view<T>(P, S, smraw);
+        if (!CACHED && tid == 0) s_scene = S;      // (read after the barriers below)
         T *X = V.tb + S.ot_x, *Y = V.tb + S.ot_y, *Z = V.tb + S.ot_z, *LAM = V.tb + S.ot_lam;
         T *YO = V.tb + S.ot_yo, *ZO = V.tb + S.ot_zo;
         T *E = V.tb + S.ot_e, *INVB = V.tb + S.ot_invb, *BT = V.tb + S.ot_b;
@@ -1674,6 +1779,15 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                 __syncthreads();
                 continue;
             }
+            // D of the subsystems that the iterations read from shared memory
+            if (S.hot_global)
+                for (int i = 0; i < S.nsub; ++i) {
+                    const SubDesc &u = P.subs[S.sub0 + i];
+                    if (u.ot_Dres < 0) continue;
+                    const VT *src = reinterpret_cast<const VT *>(V.htb + u.ot_D);
+                    VT *dst = reinterpret_cast<VT *>(V.tb + u.ot_Dres);
+                    for (int q = tid; q < u.m * u.ldd / VN; q += NT) dst[q] = src[q];
+                }
             // initial z, u = -lambda; a learned start (the launch's first step) is checked
             // after 10 iterations against the plain start's residual there, and replaced by
             // the plain start if worse
@@ -1693,7 +1807,12 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
             // constants of its item: the warp forms the items' y, and every lane of an item
             // projects it (Sec. III-C) from y gathered by shuffles, so an iteration needs one
             // block barrier (the new w) instead of two.
-            constexpr int MAXC = CachedChunks<T>::value;   // D chunks a lane keeps in registers
+            // The updates are those of grid_iter.cuh: with d = lambda' - lambda, neither y nor z is
+            // formed in the loop (z only for the stop test): 2 x chunks + 6 FP64 instructions per
+            // warp and iteration (+ 1 while the stop test fails), each of which holds the FP64 pipe for 64
+            // cycles whatever its lanes.  Contacts' two other rows are exchanged only in the warps
+            // that hold contacts, chunks beyond the warp's longest row are skipped.
+            constexpr int MAXC = cached_chunks(sizeof(T), SPLIT);
             constexpr int FSI = SPLIT == 4 ? 2 : SPLIT == 2 ? 1 : 0;
             const int xg = tid / SPLIT;
             int xt = -1, xgl = tid - xg * SPLIT, flead = 0, fslot = 0, fitem = 0;
@@ -1706,40 +1825,60 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                 fitem = fm.y >> 11;
             }
             VT dreg[MAXC];
-            bool xv = false;
-            int xwbo = 0, xnv = 0, xrow = 0, fr = 0;
-            T xc = (T)0, xbt = (T)0, xib = (T)0, xx = (T)0, yreg = (T)0, yprev = (T)0;
-            T zreg = (T)0, zprev = (T)0, lreg = (T)0;
-            RegItem<T, false> ri;
+            bool xv = false, ftwo = false, wcon = false, wsoft = false;
+            int xwbo = 0, xrow = 0, fr = 0, ftype = 0, fpart = lane, fbase = lane, wch = 0;
+            T xc = (T)0, xbt = (T)0, xib = (T)0, xe = (T)0, fa = (T)1, fmul = (T)1, fk = (T)0, fmu = (T)0;
+            T xx = (T)0, xprev = (T)0, zreg = (T)0, lreg = (T)0, lreg1 = (T)0, lreg2 = (T)0;
             auto load_cache = [&]() {
                 if (CACHED) {
 #pragma unroll
                     for (int q = 0; q < MAXC; ++q) dreg[q] = VecZero<T>::get();
                     xv = xt >= 0 && V.mlen[xt] > 0;
+                    int ch = 0;
                     if (xv) {
+                        const int xnv = (V.mlen[xt] + VN - 1) / VN;
+                        ch = (xnv + SPLIT - 1) / SPLIT;
                         xwbo = V.wbase[xt];
-                        xnv = (V.mlen[xt] + VN - 1) / VN;
                         xrow = V.row[xt];
                         xc = V.htb[V.coff[xt]];
                         xbt = BT[xt];
                         xib = INVB[xt];
                         xx = X[xt];
-                        yreg = Y[xt];
-                        yprev = yreg;
+                        xprev = xx;
                         zreg = Z[xt];
-                        zprev = zreg;
                         lreg = LAM[xrow];
-                        const VT *Dr = reinterpret_cast<const VT *>(V.htb + V.drow[xt]);
+                        lreg1 = lreg2 = lreg;
+                        const VT *Dr = d_row<T>(V, xt);
 #pragma unroll
                         for (int q = 0; q < MAXC; ++q)
                             if (xgl + q * SPLIT < xnv) dreg[q] = Dr[xgl + q * SPLIT];
+                        const Item it = V.item[fitem];
+                        const int nr = it.type == TYPE_CONTACT ? 3 : 1, side = fslot / nr;
+                        ftype = it.type;
+                        fr = fslot % nr;
+                        ftwo = it.ns > 1;
+                        fpart = (flead + ((ftwo ? side ^ 1 : side) * nr + fr) * SPLIT + xgl) & 31;
+                        fbase = (flead + side * nr * SPLIT) & 31;
+                        xe = E[xrow];
+                        fmu = MU[xrow];
+                        fk = INVS[xrow];
+                        fa = fmul = (T)1;
+                        if (ftype == TYPE_SOFT) {
+                            fa = KF[xrow] * AL[xrow] / fk;
+                            fmul = AL[xrow];
+                            fk = KF[xrow];
+                        }
+                        if (sizeof(T) == 8) { fmul *= fk; xe *= fk; }
                     }
-                    ri = RegItem<T, false>();
-                    if (xt >= 0) ri.load(V.item, V.list, fitem, INVB, E, INVS, KF, AL, MU, Z);
-                    fr = ri.nr == 3 ? fslot % 3 : 0;
+                    wch = __reduce_max_sync(0xffffffffu, ch);
+                    wcon = __any_sync(0xffffffffu, xv && ftype == TYPE_CONTACT);
+                    wsoft = __any_sync(0xffffffffu, xv && ftype == TYPE_SOFT);
                 }
             };
             load_cache();
+            // the generic variant's iterations with side-rows owned by threads (own_iter.cuh), where no
+            // thread owns more than it can keep
+            const bool owner = !CACHED && !P.stop_theta && !P.pj && S.max_sides <= 2 && S.nsr <= SUBADMM_OWN * (NT / SPLIT);
 
             int par = 0, last_par = 0, iters = 0, conv = 0, status = ST_OK;
             bool restart = false;
@@ -1747,58 +1886,126 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
             double tolc = P.tol;
             U tolb = tol_bits(T(0), tolc > 0.0 ? tolc : 0.0);
             const bool primal_stop = !P.stop_theta && P.tol > 0.0;
+            // FP64: |d| is compared with tol beta (no product); any value above the tolerance
+            // stands for a residual that is
+            const unsigned long long btol = (unsigned long long)__double_as_longlong(P.tol * (double)xbt);
+            const U btol_over = tolb + 1;
             // the loop holds no FP64 instruction in the mixed form, not even a predicated one
             // (an FP64 warp instruction issues for ~64 cycles on GB300 whatever its predicate)
             const T theta_thT = (T)P.theta_th;
+            // One iteration of this warp's side-rows: x = c + D w over each lane group (past a row's end
+            // the chunks of D are zero and those of w other rows'), the projection, the next w;
+            // with `stop` (or `all`: whole) the residual's bits
+            auto iterate = [&](const VT *wb, T *wnext, bool stop, bool all, bool first) -> U {
+                U res = 0;
+                T acc = xgl == 0 ? xc : (T)0, a1 = (T)0;
+                constexpr int QS = sizeof(T) == 4 ? 2 : 1;     // (FP32: chunks in pairs, fewer branches)
+#pragma unroll
+                for (int q = 0; q < MAXC; q += QS) {
+                    if (q >= wch) break;
+                    acc = vdot(dreg[q], wb[q * SPLIT], acc);
+                    if (QS == 2) a1 = vdot(dreg[q + QS - 1], wb[(q + QS - 1) * SPLIT], a1);
+                }
+                if (QS == 2) acc += a1;
+#pragma unroll
+                for (int o = SPLIT / 2; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                const T xo = __shfl_sync(0xffffffffu, acc, fpart);
+                // the item's sum over its sides and its lambda
+                const T g = ftwo ? acc + xo : acc;
+                T la;
+                if (sizeof(T) == 8) la = fa * lreg - (fmul * g + xe);          // (scaled by fk)
+                else if (wsoft) la = fa * lreg - (fmul * g + xe) * fk;
+                else la = lreg - (g + xe) * fk;
+                if (ftype == TYPE_HARD) la = above0(la) ? la : (T)0;
+                if (wcon) {
+                    const T l0 = __shfl_sync(0xffffffffu, la, fbase);
+                    const T l1 = __shfl_sync(0xffffffffu, la, (fbase + SPLIT) & 31);
+                    const T l2 = __shfl_sync(0xffffffffu, la, (fbase + 2 * SPLIT) & 31);
+                    if (ftype == TYPE_CONTACT) {
+                        if (!above0(l0)) {
+                            la = (T)0;
+                        } else if (fr > 0) {
+                            const T t2 = l1 * l1 + l2 * l2, lim = fmu * l0;
+                            if (above0(t2 - lim * lim)) la = la * (lim * rsq(t2));
+                        }
+                    }
+                }
+                // w of this side-row
+                const T y = xbt * acc - lreg;
+                if (xv && xgl == 0) wnext[xt] = (T)2 * la + y;
+                if (stop || all) {
+                    // |x - z| = |d| / beta, and, if no row of the warp is above the tolerance there
+                    // (FP64; always in FP32), |z - z of the iteration before|
+                    const T dl = la - lreg;
+                    bool over = false;
+                    if (sizeof(T) == 8 && !all) {
+                        over = xv && rbits(fabs(dl)) > btol;
+                        if (over) res = btol_over;
+                    }
+                    if (!__any_sync(0xffffffffu, over)) {
+                        const T dz = dl * xib, zn = acc + dz;
+                        const T zo = !first ? xx + (lreg - lreg1) * xib : zreg;
+                        if (xv && xgl == 0) res = umax(rbits(fabs(dz)), rbits(fabs(zn - zo)));
+                    }
+                }
+                xprev = xx;
+                xx = acc;
+                lreg2 = lreg1;
+                lreg1 = lreg;
+                lreg = la;
+                return res;
+            };
             int l = 0;
             pc.mark(PHASE_ASSEMBLE);
             for (;;) {
-                for (; l < P.max_iters; ++l) {
+                // a fixed iteration count: the same iteration without the tests, two at a time
+                if (CACHED && !primal_stop && !learned_mode && !P.phase && l == 0) {
+                    const VT *const wa = reinterpret_cast<const VT *>(W0 + xwbo) + xgl;
+                    const VT *const wc = reinterpret_cast<const VT *>(W1 + xwbo) + xgl;
+                    for (; l + 2 <= P.max_iters; l += 2) {
+                        iterate(wa, W1, false, false, false);
+                        __syncthreads();
+                        iterate(wc, W0, false, false, false);
+                        __syncthreads();
+                    }
+                    iters = l;
+                    last_par = 1;
+                }
+                if (!CACHED && owner) {
+                    // (a learned start's iterations up to its check on their own)
+                    const bool check = learned_mode && l <= 9 && P.max_iters > 9;
+                    const int lend = check ? 10 : P.max_iters;
+                    const OwnResult r = primal_stop
+                        ? own_iterate<T, SPLIT, NT, true>(s_scene, V.htb, l, lend, P.max_iters, par, tolb, check)
+                        : own_iterate<T, SPLIT, NT, false>(s_scene, V.htb, l, lend, P.max_iters, par, tolb, check);
+                    par ^= (r.l - l) & 1;
+                    last_par = par ^ 1;
+                    iters = r.l;
+                    conv = r.conv;
+                    l = r.conv ? r.l - 1 : r.l;
+                    pc.mark(PHASE_VSTEP);
+                    if (check && !conv) {
+                        const U mx = (U)r.mx;
+                        l = 9;
+                        if (learned && r.mx > ref10) restart = true;
+                        else {
+                            if (!learned && tid == 0) P.ref10[sc] = r.mx;
+                            if (learned && tid == 0) P.learn_skip[2 * sc + 1] = 0;     // kept: streak ends
+                            if (mx >= inf_bits(T(0))) status = ST_NAN;
+                            else if (primal_stop && mx <= tolb) conv = 1;
+                            else { l = 10; if (l < P.max_iters) continue; }
+                        }
+                    }
+                }
+                for (; (CACHED || !owner) && l < P.max_iters; ++l) {
                     // ---- v-step through the affine map x = c + D w; y = beta x - lambda
                     const T *w = par ? W1 : W0;
                     T tpart = (T)0;
                     T *wn = par ? W0 : W1;
                     U mfused = 0;
                     if (CACHED) {
-                        // x = c + D w of this side-row over its lane group
-                        T acc = (T)0;
-                        if (xv) {
-                            const VT *wb = reinterpret_cast<const VT *>(w + xwbo);
-                            T a1 = (T)0;
-#pragma unroll
-                            for (int q = 0; q < MAXC; ++q) {
-                                if (xgl + q * SPLIT < xnv) {
-                                    const VT wq = wb[xgl + q * SPLIT];
-                                    if (q & 1) a1 = vdot(dreg[q], wq, a1);
-                                    else acc = vdot(dreg[q], wq, acc);
-                                }
-                            }
-                            acc += a1;
-                        }
-#pragma unroll
-                        for (int o = SPLIT / 2; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                        const T xn = acc + xc;
-                        const T yn = xbt * xn - lreg;
-                        // the item's y (slot k on the group at lane flead + k SPLIT), its lambda,
-                        // then z, w and the residual of this side-row
-                        T ys[6], lv[3];
-#pragma unroll
-                        for (int k = 0; k < 6; ++k) ys[k] = __shfl_sync(0xffffffffu, yn, (flead + k * SPLIT) & 31);
-                        ri.lambda_of(ys, lv);
-                        const T ln = fr == 0 ? lv[0] : fr == 1 ? lv[1] : lv[2];
-                        if (xv) {
-                            const T zn = (yn + ln) * xib;
-                            if (xgl == 0) {
-                                mfused = umax(rbits(fabs(xn - zn)), rbits(fabs(zn - zreg)));
-                                wn[xt] = yn + (T)2 * ln;
-                            }
-                            zprev = zreg;
-                            zreg = zn;
-                            yprev = yreg;
-                            yreg = yn;
-                            xx = xn;
-                            lreg = ln;
-                        }
+                        mfused = iterate(reinterpret_cast<const VT *>(w + xwbo) + xgl, wn, primal_stop,
+                                         learned_mode && l == 9, l == 0);
                     } else {
                         // two side-rows per trip, two accumulators per row: independent
                         // load and FMA chains overlap
@@ -1813,7 +2020,7 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                                 mm[h] = (k + h < trips && tt[h] < S.nsr) ? V.mlen[tt[h]] : 0;
                                 T a0 = (T)0, a1 = (T)0;
                                 if (mm[h] > 0) {
-                                    const VT *Dr = reinterpret_cast<const VT *>(V.htb + V.drow[tt[h]]);
+                                    const VT *Dr = d_row<T>(V, tt[h]);
                                     const VT *wb = reinterpret_cast<const VT *>(w + V.wbase[tt[h]]);
                                     const int nv = (mm[h] + VN - 1) / VN;
                                     int c = xgl;
@@ -1938,8 +2145,9 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                         // stays non-finite (c is fixed for the step and w carries it to every
                         // coupled side-row), so the count drops to 0 or the limit ends the
                         // loop, and the step's FP64 residuals below report it
-                        const int over = __syncthreads_count(primal_stop && mloc > tolb &&
-                                                             mloc < inf_bits(T(0)));
+                        int over = 0;
+                        if (primal_stop) over = __syncthreads_count(mloc > tolb && mloc < inf_bits(T(0)));
+                        else __syncthreads();
                         par ^= 1;
                         pc.mark(PHASE_ZSTEP);
                         if (primal_stop && over == 0) { conv = 1; break; }
@@ -1979,13 +2187,16 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                     l = 0;
                     continue;
                 }
-                // the register-cached iterate: publish x, y, z, lambda (and the previous y, z)
+                // the register-cached iterate: publish x, y, z, lambda and the previous y, z (after a
+                // single iteration those are the initial ones, which init_duals left there)
                 if (CACHED && xv && xgl == 0) {
                     X[xt] = xx;
-                    Y[xt] = yreg;
-                    YO[xt] = yprev;
-                    Z[xt] = zreg;
-                    ZO[xt] = zprev;
+                    Y[xt] = xbt * xx - lreg1;
+                    Z[xt] = xx + (lreg - lreg1) * xib;
+                    if (iters > 1) {
+                        YO[xt] = xbt * xprev - lreg2;
+                        ZO[xt] = xprev + (lreg1 - lreg2) * xib;
+                    }
                     LAM[xrow] = lreg;
                 }
                 __syncthreads();
@@ -2014,8 +2225,8 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                     if (part > P.tol && l + 1 < P.max_iters) {
                         tolc *= 0.5;
                         tolb = tol_bits(T(0), tolc);
-                        if (CACHED && xv) xc = V.htb[V.coff[xt]];
-                        conv = 0;
+                        if (CACHED && xv) { xc = V.htb[V.coff[xt]]; zreg = Z[xt]; }
+                            conv = 0;
                         ++l;
                         continue;
                     }

@@ -336,14 +336,6 @@ int zeros(sim_t s, double **dst, size_t count, const char *what)
     return SIM_OK;
 }
 
-// widest row of a subsystem's envelope
-int bandwidth(const std::vector<int> &ipool, const SubDesc &u)
-{
-    int w = 0;
-    for (int p = 0; p < u.n; ++p) w = std::max(w, p - ipool[u.env_off + p]);
-    return w;
-}
-
 int iter_blocks(const sim_t s, int sms, int div);
 int iter_plan_of(sim_t s, int sc, int blocks);
 
@@ -414,6 +406,7 @@ int finalize(sim_t s)
             const HostSub &h = s->subs[sub_order[S.sub0 + i]];
             SubDesc &u = s->sdesc[S.sub0 + i];
             u.kind = h.kind; u.n = h.n; u.m = 0; u.local = i;
+            u.ot_Dres = -1;
             u.nb = h.nb;
             u.body0 = (int)(bodies.size() / SUBADMM_BODY);
             if (h.kind == KIND_RIGID) bodies.insert(bodies.end(), h.bodies.begin(), h.bodies.end());
@@ -461,8 +454,16 @@ int finalize(sim_t s)
         // subsystem's block starts on a 16-byte boundary of the iteration type (padding
         // side-rows between blocks belong to no constraint and stay zero)
         const int vn = s->opt.precision == SIM_MIXED ? 4 : 2;
+        // (the subsystems with the longest rows of D first: neighbouring side-rows, which a warp of
+        // the block kernel takes together, then have rows of about one length)
         int sr = 0;
-        for (int i = 0; i < S.nsub; ++i) {
+        std::vector<int> sub_m(S.nsub, 0), by_m(S.nsub);
+        for (int j = 0; j < S.ncon; ++j)
+            for (int q = 0; q < s->cdesc[S.con0 + j].ns; ++q)
+                sub_m[s->cdesc[S.con0 + j].sub[q]] += s->cdesc[S.con0 + j].rows;
+        for (int i = 0; i < S.nsub; ++i) by_m[i] = i;
+        std::stable_sort(by_m.begin(), by_m.end(), [&](int a, int b) { return sub_m[a] > sub_m[b]; });
+        for (int i : by_m) {
             SubDesc &u = s->sdesc[S.sub0 + i];
             sr = (sr + vn - 1) / vn * vn;
             u.sr0 = sr;
@@ -585,6 +586,8 @@ int finalize(sim_t s)
             for (int k = 0; k < n; ++k) lastr[k] = k;
             for (int r = 0; r < n; ++r)
                 for (int k = env[r]; k < r; ++k) lastr[k] = std::max(lastr[k], r);
+            u.bw = 0;
+            for (int p = 0; p < n; ++p) u.bw = std::max(u.bw, p - env[p]);
             u.env_off = (int)ipool.size();
             ipool.insert(ipool.end(), env.begin(), env.end());
             ipool.insert(ipool.end(), lastr.begin(), lastr.end());
@@ -750,7 +753,7 @@ int finalize(sim_t s)
             u.od_v = (int)sd; sd += u.n;
             u.od_id = (int)sd; sd += u.n;
             u.od_t = (int)sd; sd += u.m;
-            u.ot_L = (int)st; st += (long long)u.n * u.n;
+            u.ot_L = (int)st; st = tal(st + (long long)u.n * u.n);
             u.ot_W = (int)st; st = tal(st + (long long)((u.m + 4) / 4 * 4) * u.n);   // W: n rows
                                                                      // of m + 1 rounded up to 4
             u.ot_s = (int)st; st = tal(st + u.n);
@@ -764,7 +767,7 @@ int finalize(sim_t s)
         }
         // scene arrays (shared memory): per side-row arrays contiguous from ot_x to ot_lam
         place[sc] = Place{sd, st, sh, 2LL * S.nsub, tal((long long)S.nsr) * 9 + 6LL * S.nrow,
-                          6LL * S.nsr + 4LL * S.nitem + S.nlist};
+                          (7LL * S.nsr + 3) / 4 * 4 + 4LL * S.nitem + S.nlist};
         max_nsr = std::max(max_nsr, S.nsr);
         sr_g += S.nsr;
         rows_g += S.nrow;
@@ -780,7 +783,6 @@ int finalize(sim_t s)
     // placed there, and the others get the whole budget in a class of their own.
     const int tsize = s->opt.precision == SIM_MIXED ? 4 : 8;
     const int vn = s->opt.precision == SIM_MIXED ? 4 : 2;
-    const int chunks = s->opt.precision == SIM_MIXED ? 4 : 6;
     auto tal = [&](long long v) { return (v + vn - 1) / vn * vn; };
     const int half_budget = std::min(smem_budget, sm_smem / 2 - 2048);
     auto bytes_with = [&](const Place &q, long long d, long long tt) {
@@ -812,11 +814,22 @@ int finalize(sim_t s)
             split = mean_m >= 256 ? 32 : mean_m >= 64 ? 16 : 8;
         } else {
             while (split < 4 && 2 * split * std::max(S.nsr, 1) <= SUBADMM_THREADS) split *= 2;
+            // FP64, register-cached: the pipe is busy for 64 cycles per warp instruction whatever
+            // its lanes, so the split with the fewest instructions on a sub-partition (2 per chunk,
+            // one per halving of the sum, about 6 for the projection, times its warps)
+            int best = 1 << 30;
+            for (int q = 1; s->opt.precision == SIM_FP64 && q <= 4; q *= 2) {
+                const int nv = (sc_mpad[sc] + vn - 1) / vn;
+                if (!(sc_fmap_ok[sc] >> (q / 2) & 1) || nv > subadmm::cached_chunks(8, q) * q) continue;
+                const int warps = (q * std::max(S.nsr, 1) + 31) / 32;
+                const int cost = (warps + 3) / 4 * (2 * ((nv + q - 1) / q) + q / 2 + 6);
+                if (cost < best) { best = cost; split = q; }
+            }
         }
         if (s->split_override > 0) split = s->split_override;
         const int si = split == 4 ? 2 : split == 2 ? 1 : 0;
         const bool cached = !grid && !s->pj && s->opt.stop != SIM_STOP_THETA && (sc_fmap_ok[sc] >> si & 1) &&
-                            sc_sides[sc] <= 2 && (sc_mpad[sc] + vn - 1) / vn <= chunks * split;
+                            sc_sides[sc] <= 2 && (sc_mpad[sc] + vn - 1) / vn <= subadmm::cached_chunks(tsize, split) * split;
         const bool half = !grid && !cached && bytes_with(q, q.scd, q.sh + q.scene_t) <= half_budget;
         sc_budget[sc] = half ? half_budget : smem_budget;
         int k = 0;
@@ -831,6 +844,19 @@ int finalize(sim_t s)
         }
         s->classes[k].scenes.push_back(sc);
         sc_class[sc] = k;
+    }
+    // the scenes of a class in decreasing order of work (the entries of D, and the setup's chain of
+    // columns), so that the last blocks of a launch are short ones
+    {
+        std::vector<long long> work(nscenes, 0);
+        for (int sc = 0; sc < nscenes; ++sc)
+            for (int i = 0; i < s->scenes[sc].nsub; ++i) {
+                const SubDesc &u = s->sdesc[s->scenes[sc].sub0 + i];
+                work[sc] += (long long)u.m * u.m + 100LL * u.n;
+            }
+        for (auto &c : s->classes)
+            if (!c.grid)
+                std::stable_sort(c.scenes.begin(), c.scenes.end(), [&](int a, int b) { return work[a] > work[b]; });
     }
     for (int sc = 0; sc < nscenes; ++sc) {
         SceneDesc &S = s->scenes[sc];
@@ -851,7 +877,7 @@ int finalize(sim_t s)
                         u.m >= 16) ? 1 : 0;
                 // (FP64: by the banded factorisation)
                 if (!s->pj && s->opt.precision == SIM_FP64 && s->opt.stop != SIM_STOP_THETA && u.n >= 128 &&
-                    u.m >= 16 && bandwidth(ipool, u) <= subadmm::kBandMax)
+                    u.m >= 16 && u.bw <= subadmm::kBandMax)
                     u.tc = 1;
             }
             // everything in the workspace: the per-subsystem arrays, then the scene arrays
@@ -904,6 +930,23 @@ int finalize(sim_t s)
         S.ot_kf = (int)ot; ot += S.nrow;
         S.ot_al = (int)ot; ot += S.nrow;
         S.ot_mu = (int)ot; ot += S.nrow;
+        // D in the workspace: as many subsystems' D as fit go to shared memory for the iterations,
+        // the largest first
+        if (S.hot_global && !grid_scene) {
+            std::vector<int> ord(S.nsub);
+            for (int i = 0; i < S.nsub; ++i) ord[i] = i;
+            std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) {
+                return s->sdesc[S.sub0 + a].m > s->sdesc[S.sub0 + b].m;
+            });
+            for (int i : ord) {
+                SubDesc &u = s->sdesc[S.sub0 + i];
+                const long long at = tal(ot), end = at + (long long)u.m * u.ldd;
+                const long long tb = (od * 8 + 15) / 16 * 16, ib = (tb + end * tsize + 15) / 16 * 16;
+                if (u.m == 0 || ib + 4 * q.ints > (long long)budget) continue;
+                u.ot_Dres = (int)at;
+                ot = end;
+            }
+        }
         const long long t_base = (od * 8 + 15) / 16 * 16;
         const long long i_base = (t_base + ot * tsize + 15) / 16 * 16;
         const long long bytes = i_base + 4 * q.ints;
@@ -1457,7 +1500,7 @@ int band_plan_of(sim_t s, int sc)
     for (int i = 0; i < S.nsub; ++i) {
         const SubDesc &u = s->sdesc[S.sub0 + i];
         if (!u.tc) continue;
-        bw = std::max(bw, bandwidth(s->h_ipool, u));
+        bw = std::max(bw, u.bw);
         subadmm::BandJob J{};
         J.K = fp64 ? (void *)(sdb + u.od_L) : (void *)(stb + ts * u.ot_L);
         J.LT = stb + ts * u.ot_L;
@@ -1969,7 +2012,7 @@ namespace {
 bool cache_fits(const sim_t s, int sc, int split)
 {
     const int vn = s->opt.precision == SIM_MIXED ? 4 : 2;
-    const int chunks = s->opt.precision == SIM_MIXED ? 4 : 6;
+    const int chunks = subadmm::cached_chunks(s->opt.precision == SIM_MIXED ? 4 : 8, split);
     const int si = split == 4 ? 2 : split == 2 ? 1 : 0;
     return s->opt.stop != SIM_STOP_THETA && (s->sc_fmap_ok[sc] >> si & 1) &&
            s->sc_sides[sc] <= 2 && (s->sc_mpad[sc] + vn - 1) / vn <= chunks * split;
