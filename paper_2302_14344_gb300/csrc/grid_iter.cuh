@@ -29,7 +29,8 @@
 // reading it.  LONG = true (the large beam): a warp keeps as many rows as fit in its share of
 // the block's shared memory (33 MB over the chip) and streams the others through registers, a
 // row ahead, the first one across the barrier; the barrier's time prefetches the next rows
-// into L2.
+// into L2 (without it 64 slabs take 23.2 us an iteration instead of 17.9).  Bound by the
+// stream, some 90 MB an iteration from L2 and, for what L2 does not keep, HBM.
 #pragma once
 
 #include "grid_kernel.cuh"
@@ -202,6 +203,23 @@ __device__ __forceinline__ double2 tag_value(const TagVec &v, double2)
 {
     return make_double2(__longlong_as_double((long long)(((unsigned long long)v.a.z << 32) | v.a.x)),
                         __longlong_as_double((long long)(((unsigned long long)v.b.z << 32) | v.b.x)));
+}
+
+// A vector of a streamed D row.  A row is read once per iteration: kept out of L1, it leaves the
+// 27 KB beside the D rows in shared memory to w, which every batch of rows reads (64 slabs of 686
+// side-rows, FP32: 22.7 -> 17.9 us an iteration).
+__device__ __forceinline__ float4 load_stream(const float4 *p)
+{
+    float4 v;
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ double2 load_stream(const double2 *p)
+{
+    double2 v;
+    asm volatile("ld.global.L1::no_allocate.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p) : "memory");
+    return v;
 }
 
 // Phase tracer of the iteration kernel (see PhaseClock): in shared memory, thread 0
@@ -423,10 +441,6 @@ __global__ void __launch_bounds__(SUBADMM_ITER, 1) grid_iter_kernel(const __grid
         }
         __syncwarp();
     };
-    auto row_ptr = [&](int k) -> const VT * {      // D row of lane k's side-row
-        const int res = __shfl_sync(FULL, r_res, k), dr = __shfl_sync(FULL, r_drow, k);
-        return res >= 0 ? reinterpret_cast<const VT *>(share + res) : reinterpret_cast<const VT *>(V.htb + dr);
-    };
     load_rows();
     // initial z, u = -lambda; a learned start is checked after 10 iterations against the plain
     // start's residual there, and replaced by the plain start if worse
@@ -456,9 +470,23 @@ __global__ void __launch_bounds__(SUBADMM_ITER, 1) grid_iter_kernel(const __grid
             dst[q] = k < nv ? row[k] : VecZero<T>::get();
         }
     };
+    auto fetch_row = [&](VT *dst, int r, int nv, int seg) {       // D row of lane r's side-row
+        const int res = __shfl_sync(FULL, r_res, r), dr = __shfl_sync(FULL, r_drow, r);
+        if (res >= 0) {
+            fetch(dst, reinterpret_cast<const VT *>(share + res), nv, seg);
+            return;
+        }
+        const VT *row = reinterpret_cast<const VT *>(V.htb + dr);
+#pragma unroll
+        for (int q = 0; q < CH; ++q) {
+            const int k = (seg * CH + q) * 32 + lane;
+            dst[q] = VecZero<T>::get();
+            if (k < nv) dst[q] = load_stream(row + k);
+        }
+    };
     auto fetch_first = [&]() {
         if constexpr (LONG)
-            if (hd.nrows > 0) fetch(cur, row_ptr(0), (__shfl_sync(FULL, r_len, 0) + VN - 1) / VN, 0);
+            if (hd.nrows > 0) fetch_row(cur, 0, (__shfl_sync(FULL, r_len, 0) + VN - 1) / VN, 0);
     };
     fetch_first();
     // the tagged exchange: this launch's tags follow the last launch's (the count of iterations
@@ -579,7 +607,7 @@ __global__ void __launch_bounds__(SUBADMM_ITER, 1) grid_iter_kernel(const __grid
                                 sn = 0;
                                 nvn = kn < hd.nrows ? (__shfl_sync(FULL, r_len, kn) + VN - 1) / VN : 0;
                             }
-                            if (nvn > 0) fetch(nxt, row_ptr(kn), nvn, sn);
+                            if (nvn > 0) fetch_row(nxt, kn, nvn, sn);
                             T a = acc[r];
 #pragma unroll
                             for (int q = 0; q < CH; ++q) a = vdot(cur[q], wr[q], a);
