@@ -325,7 +325,10 @@ __global__ void __launch_bounds__(SUBADMM_ITER, 1) grid_iter_kernel(const __grid
     using U = typename VecOf<T>::U;
     constexpr int VN = VecOf<T>::N;
     constexpr bool MIXED = sizeof(T) == 4;
-    constexpr int CH = 6;                          // vectors of a row per lane and segment (LONG)
+    // vectors of a row per lane and segment (LONG): a row ahead of FP32 for the latency of its
+    // stream (3 in place of 6: 17.9 -> 21.5 us an iteration of 64 slabs); in FP64 the three buffers
+    // of 6 did not fit the registers, and 3 still cover the pipe (72k -> 47k cycles, 16 slabs)
+    constexpr int CH = MIXED ? 6 : 3;
     constexpr int RV = kWideVecs<T>();             // vectors per lane of a wide row (shape B)
     static_assert(RV <= 4, "a wide row's w is gathered at once");
     constexpr unsigned FULL = 0xffffffffu;
