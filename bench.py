@@ -245,7 +245,8 @@ class ClockSampler:
                 "samples": len(sms)}
 
 
-KERNEL_SOURCES = ("layout.h", "rigid_model.cuh", "step_kernel.cuh", "grid_kernel.cuh", "subadmm.cu")
+KERNEL_SOURCES = ("layout.h", "rigid_model.cuh", "step_kernel.cuh", "own_iter.cuh", "band_warp.cuh",
+                  "block_solve.cuh", "grid_kernel.cuh", "grid_iter.cuh", "subadmm.cu")
 
 
 def kernel_source_hash() -> str:
@@ -1098,8 +1099,8 @@ def main():
             "e2e": e2e,
             # kernels per timed launch: one per launch class, plus features, weight packing,
             # the fused network, learned duals and the two beta-scale kernels when learned
-            # (a refactorising grid scene adds its blocked factorisation's and Gram kernel's
-            # launches, which this count leaves out)
+            # (a grid scene takes a setup and an iteration launch per step and, refactorising, its
+            # factorisation's and Gram kernel's, which this count leaves out)
             "gpu_launches": len(r["launch_ms"]) * (len(r["classes"]) + (6 if learned else 0)),
             "clocks": r["clocks"],
             "launch_ms": {"mean": statistics.mean(r["launch_ms"]),

@@ -182,16 +182,20 @@ int sim_step(sim_t s, int n_steps);
  * class; classes after the first run on streams of their own forked from the simulation's
  * stream and joined back to it, so the classes overlap.
  * A scene with at least 8192 side-rows runs alone over the whole GPU instead (the grid
- * kernel: a cooperative launch whose blocks share the scene's rows, items and subsystems,
- * with two bounded grid barriers per iteration); grid classes run before the others, one
- * scene at a time, and are never captured into a graph.
+ * kernels: per step a cooperative setup launch and a cooperative iteration launch whose warps
+ * hold whole projection items, with one bounded grid barrier per iteration, or, with a fixed
+ * iteration count and small subsystems, a tagged exchange of w and no barrier; the theta stop
+ * rule and scenes with more side-rows than the grid has lanes take one launch for all steps,
+ * with two barriers per iteration); grid classes run before the others, one scene at a time,
+ * and are never captured into a graph.
  * sim_launch_classes lays the simulation out if needed and writes, for each class k <
  * max_classes, five counts at out[5k]: scenes, kernel (0 generic, 1 register-cached, 2
  * grid, 3 generic with 512 threads per block: a class whose scenes take a whole SM's shared
  * memory, so that a block has the whole register file and twice the warps), lanes per
  * side-row (1, 2 or 4; 8, 16 or 32 for the grid kernel), dynamic shared
- * memory per block in bytes (for a grid class: its staged D-row buffers at its last launch,
- * 0 before the first or without staging, see sim_grid_staging), 0.  Returns the number
+ * memory per block in bytes (for a grid class: the shared memory for its D rows at its last
+ * launch, 0 before the first, without staging, or if all its rows are short; see
+ * sim_grid_staging), 0.  Returns the number
  * of classes, or a negative SIM_E* code.
  * sim_autotune times, for each class on its own, every kernel variant that is valid for all
  * its scenes (generic with 1, 2 or 4 lanes per side-row and 256 or 512 threads per block,
@@ -253,12 +257,11 @@ int sim_step_learned(sim_t s, struct wsn_s *net, int n_steps);
  * called before the first sim_step (SIM_EINVAL after it, or for side_rows < 1). */
 int sim_grid_threshold(sim_t s, int side_rows);
 
-/* Grid kernel: with enable != 0 (the default) each warp of the warp-per-side-row v-step
- * stages its D rows in shared memory by bulk asynchronous copies (two stages per warp,
- * the next row in flight while the current one is used), when that leaves the launch its
- * blocks per SM; with 0 the rows are read from global memory directly.  The results are
- * the same either way (the same products in the same order).  Takes effect at the next
- * sim_step. */
+/* Grid kernels: with enable != 0 (the default) each warp of the iteration launch keeps as many
+ * of its long D rows in shared memory for the step as fit its share, and streams the others
+ * (the two-barrier launch: every D row staged by bulk asynchronous copies, two stages per
+ * warp); with 0 the rows are read from global memory directly.  The results are the same
+ * either way (the same products in the same order).  Takes effect at the next sim_step. */
 int sim_grid_staging(sim_t s, int enable);
 
 /* Makes linear subsystem `subsystem` co-rotational (the paper's beam model, Sec. IV-A):
@@ -291,11 +294,15 @@ int sim_set_beta_scale(sim_t s, const double *scale);
  * (SIM_EINVAL after). */
 int sim_tensor_cores(sim_t s, int enable);
 
-/* Blocked factorisation of those blocks on the tensor cores (Algorithm 1, factorise; on by
- * default; takes effect only where sim_tensor_cores is on).  A refactorised block that the
- * mixed form factorises in FP32 (not stiff by the diagonal-spread test) is factorised after
- * the setup launch instead of inside it: right-looking over panels of 128 columns, one launch
- * per panel for the diagonal tile's factor and the rows below it (CUDA cores, FP32, a thread
+/* Factorisation of those blocks after the setup launch instead of inside it (Algorithm 1,
+ * factorise; on by default; takes effect only where sim_tensor_cores is on), for refactorised
+ * blocks that the mixed form factorises in FP32 (not stiff by the diagonal-spread test).  A
+ * scene whose blocks all have narrow envelopes (at most 384 columns left of the diagonal, as FEM
+ * slabs do) takes the banded factorisation: one launch for the factors, a cluster of thread
+ * blocks per matrix, and one for W.  (The FP64 form factorises such blocks that way too, with D
+ * and c by a third launch, whatever this switch says.)  Wider envelopes, up to dense blocks, take
+ * the blocked factorisation on the tensor cores: right-looking over panels of 128 columns, one
+ * launch per panel for the diagonal tile's factor and the rows below it (CUDA cores, FP32, a thread
  * per row), and one tcgen05 launch per panel for the Schur update of the trailing tiles the
  * panel reaches inside K_i's envelope (C -= P P^T, split-TF32, accumulators in tensor
  * memory); a grid launch then solves those blocks' W before the Gram kernel.  Stiff blocks
@@ -325,8 +332,8 @@ int sim_tc_factor(sim_t s, int enable);
 #define SIM_SOLVER_PJ 1
 int sim_set_solver(sim_t s, int solver, double omega);
 
-/* Grid kernel: run the cooperative launch with `blocks` blocks (at most the resident count;
- * 0, the default, takes every resident block: 2 per SM).  Fewer blocks give each warp more
+/* Grid kernels: run the cooperative launches with `blocks` blocks (at most the resident counts;
+ * 0, the default, takes every resident block: 2 per SM in the setup, 1 in the iterations).  Fewer blocks give each warp more
  * side-rows, subsystems and items; the results do not depend on it.  Takes effect at the
  * next sim_step; SIM_EINVAL for blocks < 0. */
 int sim_grid_blocks(sim_t s, int blocks);
