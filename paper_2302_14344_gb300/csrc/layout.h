@@ -92,6 +92,8 @@ struct SubDesc {
     int gen_off;           // pool offset of A (n*n) then b (n) (generic); of mass (nb), f (n),
                            // X0 (n), K values (linear)
     int csr_off;           // linear: ipool offset of the K row pointers (n+1), then columns
+    int pat_off;           // linear: ipool offset of A's row pointers and columns (the recovery's
+                           // A v): K's, joined with the elements' node pairs if co-rotational
     int env_off;           // ipool offset of the profile of K_i: env (n), lastr (n), jlo (m), jhi (m)
     int bw;                // widest row of the envelope: largest p - env[p]
     int grp_off, ngrp;     // ipool offset of the row groups of J_ci: maximal runs of consecutive

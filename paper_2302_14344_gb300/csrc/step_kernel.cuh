@@ -1317,7 +1317,7 @@ __device__ __forceinline__ double column_jt(double out, const double *J, int n, 
 
 // v-hat of one subsystem by a whole block (see recover_v): the vector and the row groups'
 // spans in shared memory, the solves of block_solve.cuh.  A linear block's A is read through
-// K's sparse pattern (45 entries a row where the band holds 270).  1200-DOF slabs, the exit phase:
+// its sparse pattern (SubDesc::pat_off; 45 entries a row where the band holds 270).  1200-DOF slabs, the exit phase:
 // FP32 factor with refinement 10.6M -> 2.2M SM cycles, FP64 factor 5.0M -> 1.5M.
 template <typename T, int NT>
 __device__ __noinline__ void block_recover_one(const StepParams &P, const SceneDesc &S, const View<T> &V,
@@ -1369,7 +1369,7 @@ __device__ __noinline__ void block_recover_one(const StepParams &P, const SceneD
         t[r] = acc * -beta;
     }
     __syncthreads();
-    const int *rowp = P.ipool + u.csr_off, *col = rowp + n + 1;
+    const int *rowp = P.ipool + u.pat_off, *col = rowp + n + 1;
     for (int p = tid; p < n; p += NT) {
         double acc = column_jt(rhs[p], J, n, p, e.ngrp, grp, t);
         const double *Ap = Lf + (size_t)p * n;

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstddef>
+#include <iterator>
 #include <mutex>
 #include <cstdio>
 #include <cstring>
@@ -588,6 +589,31 @@ int finalize(sim_t s)
                 for (int k = env[r]; k < r; ++k) lastr[k] = std::max(lastr[k], r);
             u.bw = 0;
             for (int p = 0; p < n; ++p) u.bw = std::max(u.bw, p - env[p]);
+            // the columns of A's rows that the block recovery multiplies: K's, and for a
+            // co-rotational block the whole 3 x 3 entries of its elements' node pairs too
+            u.pat_off = u.csr_off;
+            if (u.ne > 0 && n >= SUBADMM_BIG) {
+                std::vector<std::vector<int>> nbr(u.nb);          // nodes that share an element
+                for (int el = 0; el < u.ne; ++el)
+                    for (int a = 0; a < 16; ++a)
+                        nbr[hs.tets[4 * el + a / 4]].push_back(hs.tets[4 * el + a % 4]);
+                for (auto &c : nbr) {
+                    std::sort(c.begin(), c.end());
+                    c.erase(std::unique(c.begin(), c.end()), c.end());
+                }
+                const int *rowp = hs.csr.data(), *col = rowp + n + 1;
+                std::vector<int> starts(1, 0), cols, wide;
+                for (int p = 0; p < n; ++p) {
+                    wide.clear();
+                    for (int q : nbr[p / 3])
+                        for (int r = 0; r < 3; ++r) wide.push_back(3 * q + r);
+                    std::set_union(col + rowp[p], col + rowp[p + 1], wide.begin(), wide.end(), std::back_inserter(cols));
+                    starts.push_back((int)cols.size());
+                }
+                u.pat_off = (int)ipool.size();
+                ipool.insert(ipool.end(), starts.begin(), starts.end());
+                ipool.insert(ipool.end(), cols.begin(), cols.end());
+            }
             u.env_off = (int)ipool.size();
             ipool.insert(ipool.end(), env.begin(), env.end());
             ipool.insert(ipool.end(), lastr.begin(), lastr.end());
