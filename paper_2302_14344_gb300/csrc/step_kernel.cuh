@@ -1825,20 +1825,20 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                 fitem = fm.y >> 11;
             }
             VT dreg[MAXC];
+            int woff[MAXC];                // each chunk's vector of w (past the row's end: its first)
             bool xv = false, ftwo = false, wcon = false, wsoft = false;
-            int xwbo = 0, xrow = 0, fr = 0, ftype = 0, fpart = lane, fbase = lane, wch = 0;
+            int xrow = 0, fr = 0, ftype = 0, fpart = lane, fbase = lane, wch = 0;
             T xc = (T)0, xbt = (T)0, xib = (T)0, xe = (T)0, fa = (T)1, fmul = (T)1, fk = (T)0, fmu = (T)0;
             T xx = (T)0, xprev = (T)0, zreg = (T)0, lreg = (T)0, lreg1 = (T)0, lreg2 = (T)0;
             auto load_cache = [&]() {
                 if (CACHED) {
 #pragma unroll
-                    for (int q = 0; q < MAXC; ++q) dreg[q] = VecZero<T>::get();
+                    for (int q = 0; q < MAXC; ++q) { dreg[q] = VecZero<T>::get(); woff[q] = 0; }
                     xv = xt >= 0 && V.mlen[xt] > 0;
                     int ch = 0;
                     if (xv) {
                         const int xnv = (V.mlen[xt] + VN - 1) / VN;
                         ch = (xnv + SPLIT - 1) / SPLIT;
-                        xwbo = V.wbase[xt];
                         xrow = V.row[xt];
                         xc = V.htb[V.coff[xt]];
                         xbt = BT[xt];
@@ -1850,8 +1850,11 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                         lreg1 = lreg2 = lreg;
                         const VT *Dr = d_row<T>(V, xt);
 #pragma unroll
-                        for (int q = 0; q < MAXC; ++q)
-                            if (xgl + q * SPLIT < xnv) dreg[q] = Dr[xgl + q * SPLIT];
+                        for (int q = 0; q < MAXC; ++q) {
+                            const int k = xgl + q * SPLIT;
+                            woff[q] = V.wbase[xt] / VN + (k < xnv ? k : 0);
+                            if (k < xnv) dreg[q] = Dr[k];
+                        }
                         const Item it = V.item[fitem];
                         const int nr = it.type == TYPE_CONTACT ? 3 : 1, side = fslot / nr;
                         ftype = it.type;
@@ -1894,8 +1897,8 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
             // (an FP64 warp instruction issues for ~64 cycles on GB300 whatever its predicate)
             const T theta_thT = (T)P.theta_th;
             // One iteration of this warp's side-rows: x = c + D w over each lane group (past a row's end
-            // the chunks of D are zero and those of w other rows'), the projection, the next w;
-            // with `stop` (or `all`: whole) the residual's bits
+            // a zero chunk of D meets the row's own first w: what follows in shared memory may
+            // be no number), the projection, the next w; with `stop` (or `all`: whole) the residual's bits
             auto iterate = [&](const VT *wb, T *wnext, bool stop, bool all, bool first) -> U {
                 U res = 0;
                 T acc = xgl == 0 ? xc : (T)0, a1 = (T)0;
@@ -1903,8 +1906,8 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
 #pragma unroll
                 for (int q = 0; q < MAXC; q += QS) {
                     if (q >= wch) break;
-                    acc = vdot(dreg[q], wb[q * SPLIT], acc);
-                    if (QS == 2) a1 = vdot(dreg[q + QS - 1], wb[(q + QS - 1) * SPLIT], a1);
+                    acc = vdot(dreg[q], wb[woff[q]], acc);
+                    if (QS == 2) a1 = vdot(dreg[q + QS - 1], wb[woff[q + QS - 1]], a1);
                 }
                 if (QS == 2) acc += a1;
 #pragma unroll
@@ -1960,8 +1963,7 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
             for (;;) {
                 // a fixed iteration count: the same iteration without the tests, two at a time
                 if (CACHED && !primal_stop && !learned_mode && !P.phase && l == 0) {
-                    const VT *const wa = reinterpret_cast<const VT *>(W0 + xwbo) + xgl;
-                    const VT *const wc = reinterpret_cast<const VT *>(W1 + xwbo) + xgl;
+                    const VT *const wa = reinterpret_cast<const VT *>(W0), *const wc = reinterpret_cast<const VT *>(W1);
                     for (; l + 2 <= P.max_iters; l += 2) {
                         iterate(wa, W1, false, false, false);
                         __syncthreads();
@@ -2004,7 +2006,7 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                     T *wn = par ? W0 : W1;
                     U mfused = 0;
                     if (CACHED) {
-                        mfused = iterate(reinterpret_cast<const VT *>(w + xwbo) + xgl, wn, primal_stop,
+                        mfused = iterate(reinterpret_cast<const VT *>(w), wn, primal_stop,
                                          learned_mode && l == 9, l == 0);
                     } else {
                         // two side-rows per trip, two accumulators per row: independent
