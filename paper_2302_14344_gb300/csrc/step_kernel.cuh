@@ -1891,7 +1891,9 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
             const bool primal_stop = !P.stop_theta && P.tol > 0.0;
             // FP64: |d| is compared with tol beta (no product); any value above the tolerance
             // stands for a residual that is
-            const unsigned long long btol = (unsigned long long)__double_as_longlong(P.tol * (double)xbt);
+            // (blo up to infinity, exclusive: what is not finite is not counted)
+            const unsigned long long blo = (unsigned long long)__double_as_longlong(P.tol * (double)xbt) + 1ull;
+            const unsigned long long bspan = inf_bits(0.0) - blo;
             const U btol_over = tolb + 1;
             // the loop holds no FP64 instruction in the mixed form, not even a predicated one
             // (an FP64 warp instruction issues for ~64 cycles on GB300 whatever its predicate)
@@ -1942,7 +1944,7 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                     const T dl = la - lreg;
                     bool over = false;
                     if (sizeof(T) == 8 && !all) {
-                        over = xv && rbits(fabs(dl)) > btol;
+                        over = xv && (unsigned long long)rbits(fabs(dl)) - blo < bspan;
                         if (over) res = btol_over;
                     }
                     if (!__any_sync(0xffffffffu, over)) {

@@ -1,5 +1,5 @@
 """When a step ends, in every kernel that can run it: the check of a learned start after 10
-iterations, with a fixed iteration count as well as with a tolerance."""
+iterations, with a fixed iteration count as well as with a tolerance; iterates that are not finite."""
 import numpy as np
 import pytest
 
@@ -31,3 +31,27 @@ def test_learned_start_is_judged_alike_on_grid_and_block(seed, gain):
         assert sa_["fallbacks"] == sb["fallbacks"] and sa_["total_iters"] == sb["total_iters"]
         for k in range(6):
             assert _rel(b.scene_vhat(k), a.scene_vhat(k)) < 1e-5
+
+
+@pytest.mark.parametrize("kind,precision", [("cached", 0), ("cached", 1), ("generic", 0), ("generic", 1)])
+def test_not_a_number_is_above_no_tolerance(kind, precision):
+    """With every velocity a NaN, no residual is finite and above the tolerance after the first
+    iteration: the step ends there, not at its limit, and reports SIM_ENAN."""
+    import torch
+    from paper_2302_14344_gb300 import subadmm as sa
+    p = {"cached": lambda: sg.chain(2, n_links=8, links_per_sub=2, tol_primal=1e-6, max_iters=200),
+         "generic": lambda: sg.batched(5, n_scenes=2, tol_primal=1e-6, max_iters=200)}[kind]()
+    sim = sa.Simulation(p, precision=precision)
+    assert all((c["cached"] == 1) == (kind == "cached") for c in sim.launch_classes())
+    sz = sim.sizes()
+    st = torch.empty(13 * sz["bodies"] + 6 * sz["nodes"], dtype=torch.float64).pin_memory()
+    sa.sim_read_state(sim.h, st.data_ptr())
+    st[:13 * sz["bodies"]].view(-1, 13)[:, 7:] = float("nan")
+    st[13 * sz["bodies"]:].view(-1, 6)[:, 3:] = float("nan")
+    sa.sim_write_state(sim.h, st.data_ptr())
+    sim.step(1)
+    for k in range(len(p.scenes)):
+        with pytest.raises(sa.SimError) as ei:
+            sim.residuals(k)
+        assert ei.value.code == sa.SIM_ENAN
+    assert sim.iteration_stats()["total_iters"] == len(p.scenes)
