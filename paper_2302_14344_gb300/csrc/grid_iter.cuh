@@ -340,6 +340,7 @@ __global__ void __launch_bounds__(SUBADMM_ITER, 1) grid_iter_kernel(const __grid
     __shared__ IterBarrier bar;
     __shared__ IterClock pc;
     __shared__ unsigned long long s_umax[SUBADMM_ITER / 32];
+    __shared__ int s_nan;
     GridScratch *G = P.grid;
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const int sc = P.scene_ids[0];
@@ -348,6 +349,7 @@ __global__ void __launch_bounds__(SUBADMM_ITER, 1) grid_iter_kernel(const __grid
         reinterpret_cast<int *>(&S)[q] = reinterpret_cast<const int *>(P.scenes + sc)[q];
     if (threadIdx.x == 0) {
         bar.init(G);
+        s_nan = 0;
         pc.t = clock64();
         for (int q = 0; q < 8; ++q) pc.a[q] = 0;
     }
@@ -681,12 +683,18 @@ __global__ void __launch_bounds__(SUBADMM_ITER, 1) grid_iter_kernel(const __grid
                 continue;
             }
             if (!(learned_mode && l == 9)) {
-                // the stop test rides on the barrier (see step_kernel.cuh: a non-finite iterate
-                // is not counted and is found in the step's residuals)
+                // the stop test rides on the barrier: blocks with a residual above the tolerance
+                // in the flags' low half, blocks with one that is not finite in the high half
+                // (such a step ends at once; with a fixed count the step's residuals find it)
                 unsigned over = 0;
-                if (primal_stop) over = __syncthreads_or(mloc > tolb && mloc < inf_bits(T(0))) ? 1u : 0u;
+                if (primal_stop) {
+                    if (mloc >= inf_bits(T(0))) s_nan = 1;
+                    over = __syncthreads_or(mloc > tolb) ? 1u : 0u;
+                    if (s_nan) over |= 0x10000u;
+                }
                 over = bar.sync(over);
                 pc.mark(trace, PHASE_ZSTEP);
+                if (over >> 16) { status = ST_NAN; break; }
                 if (primal_stop && over == 0) { conv = 1; break; }
                 continue;
             }

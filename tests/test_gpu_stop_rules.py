@@ -33,16 +33,20 @@ def test_learned_start_is_judged_alike_on_grid_and_block(seed, gain):
             assert _rel(b.scene_vhat(k), a.scene_vhat(k)) < 1e-5
 
 
-@pytest.mark.parametrize("kind,precision", [("cached", 0), ("cached", 1), ("generic", 0), ("generic", 1)])
+@pytest.mark.parametrize("kind,precision", [("cached", 0), ("cached", 1), ("generic", 0), ("generic", 1),
+                                            ("grid", 0), ("grid", 1), ("grid, rows streamed", 0)])
 def test_not_a_number_is_above_no_tolerance(kind, precision):
     """With every velocity a NaN, no residual is finite and above the tolerance after the first
     iteration: the step ends there, not at its limit, and reports SIM_ENAN."""
     import torch
     from paper_2302_14344_gb300 import subadmm as sa
-    p = {"cached": lambda: sg.chain(2, n_links=8, links_per_sub=2, tol_primal=1e-6, max_iters=200),
-         "generic": lambda: sg.batched(5, n_scenes=2, tol_primal=1e-6, max_iters=200)}[kind]()
-    sim = sa.Simulation(p, precision=precision)
-    assert all((c["cached"] == 1) == (kind == "cached") for c in sim.launch_classes())
+    small = kind in ("cached", "grid")
+    p = (sg.chain(2, n_links=8, links_per_sub=2, tol_primal=1e-6, max_iters=200) if small else
+         sg.batched(5, n_scenes=2, tol_primal=1e-6, max_iters=200))
+    grid = kind.startswith("grid")
+    sim = sa.Simulation(p, precision=precision, grid_side_rows=1 if grid else None)
+    sim.grid_blocks(1 if "streamed" in kind else 0)
+    assert all(c["cached"] in ([2] if grid else [1] if small else [0, 3]) for c in sim.launch_classes())
     sz = sim.sizes()
     st = torch.empty(13 * sz["bodies"] + 6 * sz["nodes"], dtype=torch.float64).pin_memory()
     sa.sim_read_state(sim.h, st.data_ptr())
