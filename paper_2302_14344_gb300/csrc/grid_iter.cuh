@@ -167,27 +167,33 @@ __device__ __forceinline__ T reduce8(T *a)
     return a[0];
 }
 
-// One w of the tagged exchange: value and tag in 8 bytes (FP32), or two such halves (FP64), and
-// a vector's worth of them (32 bytes) read at once
+// One w of the tagged exchange: value and tag in one 64-bit word (FP32), or the value's halves in
+// two (FP64), and a vector's worth of them (32 bytes) read at once.  Each 64-bit element of an
+// access is read and written whole, so a tag never comes without its value.
 __device__ __forceinline__ void tag_store(void *p, float v, unsigned tag)
 {
-    asm volatile("st.relaxed.gpu.global.v2.u32 [%0], {%1, %2};" ::"l"(p), "r"(__float_as_uint(v)), "r"(tag) : "memory");
+    asm volatile("{\n\t.reg .b64 a;\n\tmov.b64 a, {%1, %2};\n\tst.relaxed.gpu.global.b64 [%0], a;\n\t}"
+                 ::"l"(p), "r"(__float_as_uint(v)), "r"(tag) : "memory");
 }
 __device__ __forceinline__ void tag_store(void *p, double v, unsigned tag)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    asm volatile("st.relaxed.gpu.global.v4.u32 [%0], {%1, %2, %3, %2};"
+    asm volatile("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %2};\n\t"
+                 "st.relaxed.gpu.global.v2.b64 [%0], {a, b};\n\t}"
                  ::"l"(p), "r"((unsigned)b), "r"(tag), "r"((unsigned)(b >> 32)) : "memory");
 }
 struct TagVec { uint4 a, b; };
+__device__ __forceinline__ uint4 tag_load2(const void *p)
+{
+    uint4 v;
+    asm volatile("{\n\t.reg .b64 a, b;\n\tld.relaxed.gpu.global.v2.b64 {a, b}, [%4];\n\t"
+                 "mov.b64 {%0, %1}, a;\n\tmov.b64 {%2, %3}, b;\n\t}"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ TagVec tag_load(const void *p)
 {
-    TagVec v;
-    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.a.x), "=r"(v.a.y), "=r"(v.a.z), "=r"(v.a.w) : "l"(p) : "memory");
-    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.b.x), "=r"(v.b.y), "=r"(v.b.z), "=r"(v.b.w) : "l"((const char *)p + 16) : "memory");
-    return v;
+    return TagVec{tag_load2(p), tag_load2((const char *)p + 16)};
 }
 // every word is of iteration `tag`, or padding (no owner; the host sets its tag to ~0)
 __device__ __forceinline__ bool tag_ready(const TagVec &v, unsigned tag)
