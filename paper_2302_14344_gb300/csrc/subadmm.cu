@@ -884,6 +884,19 @@ int finalize(sim_t s)
             if (!c.grid)
                 std::stable_sort(c.scenes.begin(), c.scenes.end(), [&](int a, int b) { return work[a] > work[b]; });
     }
+    // Classes whose scenes with D in the workspace copy it to the shared memory that is left, for the
+    // iterations.  That takes L1 from the setup, whose one-warp factorisations of wide bands
+    // live on it (2 slabs of 360 DOF: 33.5M -> 71M cycles), so no scene of the class may hold
+    // such a block; and in FP64 the iterations are bound by the FP64 pipe, with L1 enough to feed
+    // it (12 uneven scenes: 22.8k cycles an iteration without the copy, 26.9k with it; FP32, 384
+    // scenes: 6.8k without, 4.5k with).
+    std::vector<char> keep_D(s->classes.size(), s->opt.precision == SIM_MIXED ? 1 : 0);
+    for (int sc = 0; sc < nscenes; ++sc) {
+        const Place &q = place[sc];
+        if (bytes_with(q, q.scd, q.sh + q.scene_t) <= (long long)sc_budget[sc]) continue;
+        for (int i = 0; i < s->scenes[sc].nsub; ++i)
+            if (s->sdesc[s->scenes[sc].sub0 + i].bw > subadmm::kNarrowBand) keep_D[sc_class[sc]] = 0;
+    }
     for (int sc = 0; sc < nscenes; ++sc) {
         SceneDesc &S = s->scenes[sc];
         const Place &q = place[sc];
@@ -956,9 +969,9 @@ int finalize(sim_t s)
         S.ot_kf = (int)ot; ot += S.nrow;
         S.ot_al = (int)ot; ot += S.nrow;
         S.ot_mu = (int)ot; ot += S.nrow;
-        // D in the workspace: as many subsystems' D as fit go to shared memory for the iterations,
-        // the largest first
-        if (S.hot_global && !grid_scene) {
+        // D in the workspace: as many subsystems' D as fit go to shared memory for the iterations
+        // (keep_D, above), the largest first
+        if (S.hot_global && !grid_scene && keep_D[sc_class[sc]]) {
             std::vector<int> ord(S.nsub);
             for (int i = 0; i < S.nsub; ++i) ord[i] = i;
             std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) {
