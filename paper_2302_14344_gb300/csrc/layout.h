@@ -52,6 +52,9 @@ struct SceneDesc {
     int fmap_off[3];
     // grid kernel: bytes of one staged D row (the longest row, whole 16-byte vectors)
     int row_bytes;
+    // block kernel, side-rows owned by threads: ipool offset of, per side-row, the side-row of the
+    // same row on the constraint's other side + 1 (0: none) | type << 16 | row of its contact << 18
+    int own_off;
     int item_g0, list_g0;  // global offsets of the scene's item / list tables
     int nasm, asm_g0;      // assembly slots (constraint indices grouped by kind, -1 = idle)
     // ipool offset of three prefix sums over the subsystems (nsub + 1 each): chunks of 32

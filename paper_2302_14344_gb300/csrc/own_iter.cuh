@@ -24,11 +24,12 @@ struct OwnResult {
     unsigned long long mx;     // asked for: the largest residual's bits of the last iteration
 };
 
-// Iterations l .. lend - 1 of the scene whose descriptor and shared arrays these are; par: which of
+// Iterations l .. lend - 1 of the scene whose descriptor and shared arrays these are (map: see
+// SceneDesc::own_off); par: which of
 // the two w holds iteration l's.  STOP: ends when no residual is above tolb.  max_iters: the step's
 // limit (its last two iterations keep z and y).
 template <typename T, int SPLIT, int NT, bool STOP>
-__device__ __noinline__ OwnResult own_iterate(const SceneDesc &S, const T *htb, int l, int lend, int max_iters,
+__device__ __noinline__ OwnResult own_iterate(const SceneDesc &S, const T *htb, const int *map, int l, int lend, int max_iters,
                                               int par, typename VecOf<T>::U tolb, bool want_max)
 {
     using VT = typename VecOf<T>::V;
@@ -61,7 +62,7 @@ __device__ __noinline__ OwnResult own_iterate(const SceneDesc &S, const T *htb, 
         o.kind = 16;
         o.bt = o.c = o.e = o.fk = o.lam = (T)0;
         if (t >= nsr || ib[5 * nsr + t] == 0) continue;
-        const int meta = ib[6 * nsr + t], dr = ib[2 * nsr + t], type = meta >> 16 & 3;
+        const int meta = map[t], dr = ib[2 * nsr + t], type = meta >> 16 & 3;
         o.nv = (ib[5 * nsr + t] + VN - 1) / VN;
         o.w = ib[4 * nsr + t];
         o.row = ib[t];

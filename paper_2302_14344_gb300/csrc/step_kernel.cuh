@@ -170,7 +170,6 @@ struct View {
     T *htb;              // per-subsystem iteration arrays (D, c): shared memory unless the
                          // scene cannot hold even those
     int *row, *sub, *drow, *coff, *wbase, *mlen;   // per side-row tables
-    int *meta;           // other side's side-row of the row + 1 | type << 16 | row of its contact << 18
     Item *item;
     int *list;
 };
@@ -197,9 +196,8 @@ __device__ View<T> scene_view(const StepParams &P, const SceneDesc &S, unsigned 
     V.coff = ib + 3 * S.nsr;
     V.wbase = ib + 4 * S.nsr;
     V.mlen = ib + 5 * S.nsr;
-    V.meta = ib + 6 * S.nsr;
-    V.item = reinterpret_cast<Item *>(ib + (7 * S.nsr + 3) / 4 * 4);
-    V.list = ib + (7 * S.nsr + 3) / 4 * 4 + 4 * S.nitem;
+    V.item = reinterpret_cast<Item *>(ib + 6 * S.nsr);
+    V.list = ib + 6 * S.nsr + 4 * S.nitem;
     return V;
 }
 
@@ -297,7 +295,6 @@ __device__ void scene_tables(const StepParams &P, const SceneDesc &S, const View
 {
     for (int t = d.tid; t < S.nsr; t += d.nthreads) {
         V.row[t] = 0; V.sub[t] = 0; V.drow[t] = 0; V.coff[t] = 0; V.wbase[t] = 0; V.mlen[t] = 0;
-        V.meta[t] = 0;
     }
     d.sync();
     for (int j = d.tid; j < S.ncon; j += d.nthreads) {
@@ -313,7 +310,6 @@ __device__ void scene_tables(const StepParams &P, const SceneDesc &S, const View
                 V.coff[t] = u.ot_c + lr;
                 V.wbase[t] = u.sr0;
                 V.mlen[t] = u.m;
-                V.meta[t] = (c.ns == 2 ? c.sr[s ^ 1] + r + 1 : 0) | c.type << 16 | (c.type == TYPE_CONTACT ? r << 18 : 0);
             }
         }
     }
@@ -1980,8 +1976,8 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                     const bool check = learned_mode && l <= 9 && P.max_iters > 9;
                     const int lend = check ? 10 : P.max_iters;
                     const OwnResult r = primal_stop
-                        ? own_iterate<T, SPLIT, NT, true>(s_scene, V.htb, l, lend, P.max_iters, par, tolb, check)
-                        : own_iterate<T, SPLIT, NT, false>(s_scene, V.htb, l, lend, P.max_iters, par, tolb, check);
+                        ? own_iterate<T, SPLIT, NT, true>(s_scene, V.htb, P.ipool + S.own_off, l, lend, P.max_iters, par, tolb, check)
+                        : own_iterate<T, SPLIT, NT, false>(s_scene, V.htb, P.ipool + S.own_off, l, lend, P.max_iters, par, tolb, check);
                     par ^= (r.l - l) & 1;
                     last_par = par ^ 1;
                     iters = r.l;

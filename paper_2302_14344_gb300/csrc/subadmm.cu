@@ -673,6 +673,18 @@ int finalize(sim_t s)
                 ipool.push_back(acc);
             }
         }
+        // side-rows owned by threads (scenes that the block kernel may take that way)
+        S.own_off = (int)ipool.size();
+        if (S.nsr <= SUBADMM_OWN * SUBADMM_WIDE) {
+            ipool.resize(ipool.size() + S.nsr, 0);
+            for (int j = 0; j < S.ncon; ++j) {
+                const ConDesc &c = s->cdesc[S.con0 + j];
+                for (int q = 0; q < c.ns; ++q)
+                    for (int r = 0; r < c.rows; ++r)
+                        ipool[S.own_off + c.sr[q] + r] = (c.ns == 2 ? c.sr[q ^ 1] + r + 1 : 0) | c.type << 16 |
+                                                         (c.type == TYPE_CONTACT ? r << 18 : 0);
+            }
+        }
         // z-step items: one per row of an equality / hard / soft constraint, one per contact;
         // ordered by type so that neighbouring threads run the same projection
         S.item_g0 = (int)items.size();
@@ -779,9 +791,9 @@ int finalize(sim_t s)
             u.od_v = (int)sd; sd += u.n;
             u.od_id = (int)sd; sd += u.n;
             u.od_t = (int)sd; sd += u.m;
+            // W: n rows of m + 1 rounded up to 4; then L (both start on 16 bytes)
+            u.ot_W = (int)st; st += (long long)((u.m + 4) / 4 * 4) * u.n;
             u.ot_L = (int)st; st = tal(st + (long long)u.n * u.n);
-            u.ot_W = (int)st; st = tal(st + (long long)((u.m + 4) / 4 * 4) * u.n);   // W: n rows
-                                                                     // of m + 1 rounded up to 4
             u.ot_s = (int)st; st = tal(st + u.n);
             // D rows are ldd apart: an odd number of 16-byte vectors, so the rows that the
             // lanes of a warp read at once fall in different shared-memory banks
@@ -793,7 +805,7 @@ int finalize(sim_t s)
         }
         // scene arrays (shared memory): per side-row arrays contiguous from ot_x to ot_lam
         place[sc] = Place{sd, st, sh, 2LL * S.nsub, tal((long long)S.nsr) * 9 + 6LL * S.nrow,
-                          (7LL * S.nsr + 3) / 4 * 4 + 4LL * S.nitem + S.nlist};
+                          6LL * S.nsr + 4LL * S.nitem + S.nlist};
         max_nsr = std::max(max_nsr, S.nsr);
         sr_g += S.nsr;
         rows_g += S.nrow;

@@ -24,3 +24,12 @@ def test_D_is_copied_only_where_the_setup_does_not_need_the_cache():
         assert far and all((b > 200000) == (precision == 1) for b in far), far
         sim, info = _sim(beam, precision)
         assert info[0]["placement"] == 2 and info[0]["smem_bytes"] < 90000, info
+
+
+def test_setup_arrays_stay_on_chip():
+    """Tables that only the iterations' start reads take no shared memory: scenes of dense blocks a few
+    bytes below half an SM's shared memory keep all of their arrays there."""
+    p = sg.generic(3, n_scenes=16, n_sub=5, n_range=(1, 42), extra=6, tol_primal=-1, max_iters=10)
+    sim, info = _sim(p, 1)
+    assert [i["placement"] for i in info] == [0] * 16, info
+    assert max(i["smem_bytes"] for i in info) > 110000
