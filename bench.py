@@ -245,7 +245,7 @@ class ClockSampler:
                 "samples": len(sms)}
 
 
-KERNEL_SOURCES = ("layout.h", "rigid_model.cuh", "step_kernel.cuh", "own_iter.cuh", "band_warp.cuh",
+KERNEL_SOURCES = ("layout.h", "rigid_model.cuh", "step_kernel.cuh", "own_iter.cuh", "item_iter.cuh", "band_warp.cuh",
                   "block_solve.cuh", "grid_kernel.cuh", "grid_iter.cuh", "subadmm.cu")
 
 

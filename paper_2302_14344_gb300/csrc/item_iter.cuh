@@ -11,18 +11,14 @@
 namespace subadmm {
 
 // what decides the projection and the end of the step
-template <typename T>
-struct ItemRule {
-    int pj, stop_theta;
-    bool primal_stop, trace;
-    T pj_omega, theta_th;
-};
+enum { ITEM_PJ = 1, ITEM_THETA = 2, ITEM_TOL = 4, ITEM_TRACE = 8 };
 
 // Iterations l .. lend - 1 of the scene whose descriptor and shared arrays these are; par: which of
-// the two w holds iteration l's; want_max: the residual of iteration lend - 1 is returned, not tested
+// the two w holds iteration l's; rule: ITEM_*; want_max: the residual of iteration lend - 1 is
+// returned, not tested
 template <typename T, int SPLIT, int NT>
-__device__ __noinline__ IterResult item_iterate(const SceneDesc &S, const T *htb, ItemRule<T> rule, int l, int lend,
-                                                int par, typename VecOf<T>::U tolb, bool want_max)
+__device__ __noinline__ IterResult item_iterate(const SceneDesc &S, const T *htb, int rule, T pj_omega, T theta_th,
+                                                int l, int lend, int par, typename VecOf<T>::U tolb, bool want_max)
 {
     using VT = typename VecOf<T>::V;
     using U = typename VecOf<T>::U;
@@ -44,6 +40,7 @@ __device__ __noinline__ IterResult item_iterate(const SceneDesc &S, const T *htb
     const int w0 = S.ot_w0, w1 = S.ot_w1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int xg = tid / SPLIT, xgl = tid - xg * SPLIT, trips = (nsr + groups - 1) / groups;
+    const bool stop_theta = rule & ITEM_THETA;
     IterResult res{l, 0, par, par, 0ull, 0.0, 0ll};
     for (; l < lend; ++l) {
         const T *const w = tb + (par ? w1 : w0);
@@ -83,7 +80,7 @@ __device__ __noinline__ IterResult item_iterate(const SceneDesc &S, const T *htb
                 if (mm[h] > 0 && xgl == 0) {
                     const T a = acc[h] + htb[coff[t]];
                     const T ynew = BT[t] * a - LAM[row[t]];
-                    if (rule.stop_theta) {
+                    if (stop_theta) {
                         const T d = ynew - Y[t];
                         tpart += d * d;
                     }
@@ -93,16 +90,16 @@ __device__ __noinline__ IterResult item_iterate(const SceneDesc &S, const T *htb
                 }
             }
         }
-        if (rule.stop_theta) {
+        if (stop_theta) {
 #pragma unroll
             for (int o = 16; o; o >>= 1) tpart += __shfl_xor_sync(0xffffffffu, tpart, o);
             if (lane == 0) tred[l & 1][warp] = tpart;
         }
         __syncthreads();
-        if (rule.stop_theta) {
+        if (stop_theta) {
             T ths = (T)0;
             for (int q = 0; q < NW; ++q) ths += tred[l & 1][q];
-            if (l >= 1 && ths < rule.theta_th) {
+            if (l >= 1 && ths < theta_th) {
                 // (before the z-step: w is that of this v-step)
                 res.theta = (double)ths;
                 res.conv = 1;
@@ -111,15 +108,15 @@ __device__ __noinline__ IterResult item_iterate(const SceneDesc &S, const T *htb
                 return res;
             }
         }
-        const long long t0 = rule.trace ? clock64() : 0ll;
+        const long long t0 = rule & ITEM_TRACE ? clock64() : 0ll;
         // ---- z-step (Sec. III-C); u = -lambda; max(|x - z|, |dz|) as bits
         U mloc = 0;
         for (int i = tid; i < nitem; i += NT) {
             const Item it = item[i];
             if (it.type < 0) continue;
             const int *ls = list + it.lo;
-            if (rule.pj) {
-                mloc = pj_item<T, U>(it, ls, X, E, INVS, KF, AL, MU, LAM, Z, ZO, wn, rule.pj_omega, mloc);
+            if (rule & ITEM_PJ) {
+                mloc = pj_item<T, U>(it, ls, X, E, INVS, KF, AL, MU, LAM, Z, ZO, wn, pj_omega, mloc);
                 continue;
             }
             if (it.type == TYPE_CONTACT) {
@@ -187,11 +184,11 @@ __device__ __noinline__ IterResult item_iterate(const SceneDesc &S, const T *htb
         } else {
             // (the stop test rides on the barrier, see step_kernel)
             int over = 1;
-            if (rule.primal_stop) over = __syncthreads_count(mloc > tolb && mloc < inf_bits(T(0)));
+            if (rule & ITEM_TOL) over = __syncthreads_count(mloc > tolb && mloc < inf_bits(T(0)));
             else __syncthreads();
             if (over == 0) res.conv = 1;
         }
-        if (rule.trace) res.z_cycles += clock64() - t0;
+        if (rule & ITEM_TRACE) res.z_cycles += clock64() - t0;
         if (res.conv) { ++l; break; }
     }
     res.l = l;

@@ -18,10 +18,14 @@
 
 namespace subadmm {
 
-struct OwnResult {
+// of own_iterate and item_iterate (item_iter.cuh)
+struct IterResult {
     int l;                     // iterations run so far
     int conv;                  // 1: the stop test held in iteration l - 1
+    int par, last_par;         // which w the next iteration reads, which one the last one read
     unsigned long long mx;     // asked for: the largest residual's bits of the last iteration
+    double theta;              // theta of the last iteration (its stop rule)
+    long long z_cycles;        // traced: cycles of the z-steps
 };
 
 // Iterations l .. lend - 1 of the scene whose descriptor and shared arrays these are (map: see
@@ -29,7 +33,7 @@ struct OwnResult {
 // the two w holds iteration l's.  STOP: ends when no residual is above tolb.  max_iters: the step's
 // limit (its last two iterations keep z and y).
 template <typename T, int SPLIT, int NT, bool STOP>
-__device__ __noinline__ OwnResult own_iterate(const SceneDesc &S, const T *htb, const int *map, int l, int lend, int max_iters,
+__device__ __noinline__ IterResult own_iterate(const SceneDesc &S, const T *htb, const int *map, int l, int lend, int max_iters,
                                               int par, typename VecOf<T>::U tolb, bool want_max)
 {
     using VT = typename VecOf<T>::V;
@@ -78,7 +82,7 @@ __device__ __noinline__ OwnResult own_iterate(const SceneDesc &S, const T *htb, 
         con = con || type == TYPE_CONTACT;
     }
     con = __any_sync(0xffffffffu, con);
-    OwnResult res{l, 0, 0ull};
+    IterResult res{l, 0, 0, 0, 0ull, 0.0, 0ll};
     for (; l < lend; ++l) {
         const int wc = par ? w1 : w0, wn = par ? w0 : w1;
         // ---- v-step
@@ -183,6 +187,8 @@ __device__ __noinline__ OwnResult own_iterate(const SceneDesc &S, const T *htb, 
         if (ow[k].nv > 0 && xgl == 0) LAM[ow[k].row] = ow[k].lam;
     __syncthreads();
     res.l = l;
+    res.par = par;
+    res.last_par = par ^ 1;
     return res;
 }
 

@@ -149,6 +149,11 @@ struct PhaseClock {
             t = when;
         }
     }
+    __device__ __forceinline__ void move(int from, int to, long long cycles)
+    {
+        a[from] -= cycles;
+        a[to] += cycles;
+    }
     __device__ __forceinline__ void flush(int iters, int steps = 1)
     {
         if (out) {
@@ -1486,17 +1491,19 @@ __device__ void recover_v(const StepParams &P, const SceneDesc &S, const View<T>
     }
 }
 
-// The block kernel's once-per-step phases as calls (arguments by value), so that the
-// register allocation of its iteration loop is not shaped by the setup code's.
+// The block kernel's once-per-step phases as calls, so that the register allocation of its
+// iteration loop is not shaped by the setup code's.  The parameters and the scene's descriptor stay
+// where they are (parameter and shared memory): by value they took 500 bytes of every thread's
+// frame, through the L1 that the setup lives on, and registers across the calls.
 template <typename T>
-__device__ __noinline__ long long block_setup(StepParams P, SceneDesc S, View<T> V, int *status,
+__device__ __noinline__ long long block_setup(const StepParams &P, const SceneDesc &S, View<T> V, int *status,
                                               int step)
 {
     return scene_setup<T>(P, S, V, status, step, BlockDist());
 }
 
 template <typename T>
-__device__ __noinline__ void block_recover(StepParams P, SceneDesc S, View<T> V, const T *w)
+__device__ __noinline__ void block_recover(const StepParams &P, const SceneDesc &S, View<T> V, const T *w)
 {
     recover_v<T>(P, S, V, w, BlockDist());
 }
@@ -1574,6 +1581,10 @@ __device__ __forceinline__ U pj_item(const Item &it, const int *ls, const T *X, 
     }
     return mloc;
 }
+
+}  // namespace subadmm
+#include "item_iter.cuh"
+namespace subadmm {
 
 // One z-step item held in a thread's registers for a whole step (items with at most two
 // sides): its type, row, side-rows and the step's constants.  KEEP_Z: the z of its
@@ -1726,7 +1737,7 @@ struct RegItem {
 // whose scenes take a whole SM's shared memory (one block per SM), which then uses the whole
 // register file and twice the warps per scene
 template <typename T, int SPLIT, bool CACHED, int NT = SUBADMM_THREADS>
-__global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) step_kernel(StepParams P)
+__global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) step_kernel(const __grid_constant__ StepParams P)
 {
     static_assert(!CACHED || NT == SUBADMM_THREADS, "the register-cached map is laid out for 256 threads");
     constexpr int NW = NT / 32;
@@ -1735,18 +1746,20 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
     constexpr int VN = VecOf<T>::N;
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ double red[4][SUBADMM_MAXWARPS];
-    __shared__ U ured[2][NW];
-    __shared__ T tred[2][NW];
+    __shared__ U ured[NW];
     __shared__ int s_status;
-    __shared__ SceneDesc s_scene;          // (own_iterate)
+    __shared__ SceneDesc s_scene;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr bool MIXED = sizeof(T) == 4;
 
     for (int k = blockIdx.x; k < P.nscenes; k += gridDim.x) {
         const int sc = P.scene_ids[k];
-        const SceneDesc S = P.scenes[sc];
+        __syncthreads();                           // (the scene before this one is done)
+        for (int q = tid; q < (int)(sizeof(SceneDesc) / 4); q += NT)
+            reinterpret_cast<int *>(&s_scene)[q] = reinterpret_cast<const int *>(P.scenes + sc)[q];
+        __syncthreads();
+        const SceneDesc &S = s_scene;
         const View<T> V = scene_view<T>(P, S, smraw);
-        if (!CACHED && tid == 0) s_scene = S;      // (read after the barriers below)
         T *X = V.tb + S.ot_x, *Y = V.tb + S.ot_y, *Z = V.tb + S.ot_z, *LAM = V.tb + S.ot_lam;
         T *YO = V.tb + S.ot_yo, *ZO = V.tb + S.ot_zo;
         T *E = V.tb + S.ot_e, *INVB = V.tb + S.ot_invb, *BT = V.tb + S.ot_b;
@@ -1893,7 +1906,8 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
             const U btol_over = tolb + 1;
             // the loop holds no FP64 instruction in the mixed form, not even a predicated one
             // (an FP64 warp instruction issues for ~64 cycles on GB300 whatever its predicate)
-            const T theta_thT = (T)P.theta_th;
+            const int rule = (P.pj ? ITEM_PJ : 0) | (P.stop_theta ? ITEM_THETA : 0) | (primal_stop ? ITEM_TOL : 0) |
+                             (P.phase ? ITEM_TRACE : 0);
             // One iteration of this warp's side-rows: x = c + D w over each lane group (past a row's end
             // a zero chunk of D meets the row's own first w: what follows in shared memory may
             // be no number), the projection, the next w; with `stop` (or `all`: whole) the residual's bits
@@ -1971,19 +1985,25 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                     iters = l;
                     last_par = 1;
                 }
-                if (!CACHED && owner) {
+                if constexpr (!CACHED) {
                     // (a learned start's iterations up to its check on their own)
                     const bool check = learned_mode && l <= 9 && P.max_iters > 9;
                     const int lend = check ? 10 : P.max_iters;
-                    const OwnResult r = primal_stop
-                        ? own_iterate<T, SPLIT, NT, true>(s_scene, V.htb, P.ipool + S.own_off, l, lend, P.max_iters, par, tolb, check)
-                        : own_iterate<T, SPLIT, NT, false>(s_scene, V.htb, P.ipool + S.own_off, l, lend, P.max_iters, par, tolb, check);
-                    par ^= (r.l - l) & 1;
-                    last_par = par ^ 1;
+                    IterResult r;
+                    if (!owner)
+                        r = item_iterate<T, SPLIT, NT>(s_scene, V.htb, rule, (T)P.pj_omega, (T)P.theta_th, l, lend, par, tolb, check);
+                    else if (primal_stop)
+                        r = own_iterate<T, SPLIT, NT, true>(s_scene, V.htb, P.ipool + S.own_off, l, lend, P.max_iters, par, tolb, check);
+                    else
+                        r = own_iterate<T, SPLIT, NT, false>(s_scene, V.htb, P.ipool + S.own_off, l, lend, P.max_iters, par, tolb, check);
+                    par = r.par;
+                    last_par = r.last_par;
                     iters = r.l;
                     conv = r.conv;
+                    if (r.conv && P.stop_theta) th = r.theta;
                     l = r.conv ? r.l - 1 : r.l;
                     pc.mark(PHASE_VSTEP);
+                    pc.move(PHASE_VSTEP, PHASE_ZSTEP, r.z_cycles);
                     if (check && !conv) {
                         const U mx = (U)r.mx;
                         l = 9;
@@ -1997,148 +2017,13 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                         }
                     }
                 }
-                for (; (CACHED || !owner) && l < P.max_iters; ++l) {
-                    // ---- v-step through the affine map x = c + D w; y = beta x - lambda
-                    const T *w = par ? W1 : W0;
-                    T tpart = (T)0;
-                    T *wn = par ? W0 : W1;
-                    U mfused = 0;
-                    if (CACHED) {
-                        mfused = iterate(reinterpret_cast<const VT *>(w), wn, primal_stop,
-                                         learned_mode && l == 9, l == 0);
-                    } else {
-                        // two side-rows per trip, two accumulators per row: independent
-                        // load and FMA chains overlap
-                        constexpr int groups = NT / SPLIT;
-                        const int trips = (S.nsr + groups - 1) / groups;
-                        for (int k = 0; k < trips; k += 2) {
-                            int tt[2], mm[2];
-                            T acc[2];
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                tt[h] = xg + (k + h) * groups;
-                                mm[h] = (k + h < trips && tt[h] < S.nsr) ? V.mlen[tt[h]] : 0;
-                                T a0 = (T)0, a1 = (T)0;
-                                if (mm[h] > 0) {
-                                    const VT *Dr = d_row<T>(V, tt[h]);
-                                    const VT *wb = reinterpret_cast<const VT *>(w + V.wbase[tt[h]]);
-                                    const int nv = (mm[h] + VN - 1) / VN;
-                                    int c = xgl;
-                                    for (; c + SPLIT < nv; c += 2 * SPLIT) {
-                                        a0 = vdot(Dr[c], wb[c], a0);
-                                        a1 = vdot(Dr[c + SPLIT], wb[c + SPLIT], a1);
-                                    }
-                                    if (c < nv) a0 = vdot(Dr[c], wb[c], a0);
-                                }
-                                acc[h] = a0 + a1;
-                            }
-#pragma unroll
-                            for (int o = SPLIT / 2; o; o >>= 1) {
-                                acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
-                                acc[1] += __shfl_xor_sync(0xffffffffu, acc[1], o);
-                            }
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const int t = tt[h];
-                                if (mm[h] > 0 && xgl == 0) {
-                                    const T a = acc[h] + V.htb[V.coff[t]];
-                                    const T ynew = BT[t] * a - LAM[V.row[t]];
-                                    if (P.stop_theta) {
-                                        const T d = ynew - Y[t];
-                                        tpart += d * d;
-                                    }
-                                    YO[t] = Y[t];
-                                    Y[t] = ynew;
-                                    X[t] = a;
-                                }
-                            }
-                        }
-                    }
-                    if (!CACHED) {
-                        if (P.stop_theta) {
-#pragma unroll
-                            for (int o = 16; o; o >>= 1) tpart += __shfl_xor_sync(0xffffffffu, tpart, o);
-                            if (lane == 0) tred[l & 1][warp] = tpart;
-                        }
-                        __syncthreads();
-                    }
+                for (; CACHED && l < P.max_iters; ++l) {
+                    // x = c + D w, the projection and the next w (iterate, above)
+                    const U mloc = iterate(reinterpret_cast<const VT *>(par ? W1 : W0), par ? W0 : W1, primal_stop,
+                                           learned_mode && l == 9, l == 0);
                     pc.mark(PHASE_VSTEP);
                     last_par = par;
                     iters = l + 1;
-                    if (!CACHED && P.stop_theta) {
-                        T ths = (T)0;
-                        for (int q = 0; q < NW; ++q) ths += tred[l & 1][q];
-                        if (l >= 1 && ths < theta_thT) { th = (double)ths; conv = 1; break; }
-                    }
-                    // ---- z-step (Sec. III-C); u = -lambda; max(|x - z|, |dz|) as bits
-                    U mloc = 0;
-                    if (CACHED) {
-                        mloc = mfused;
-                    } else {
-                        for (int i = tid; i < S.nitem; i += NT) {
-                            const Item it = V.item[i];
-                            if (it.type < 0) continue;
-                            const int *ls = V.list + it.lo;
-                            if (P.pj) {
-                                mloc = pj_item<T, U>(it, ls, X, E, INVS, KF, AL, MU, LAM, Z, ZO,
-                                                     wn, (T)P.pj_omega, mloc);
-                                continue;
-                            }
-                            if (it.type == TYPE_CONTACT) {
-                                T q0 = (T)0, q1 = (T)0, q2 = (T)0;
-                                for (int s = 0; s < it.ns; ++s) {
-                                    const int t = ls[s];
-                                    const T ib = INVB[t];
-                                    q0 += Y[t] * ib; q1 += Y[t + 1] * ib; q2 += Y[t + 2] * ib;
-                                }
-                                const T is = INVS[it.row];
-                                const T ln = -(q0 + E[it.row]) * is;
-                                const T l1 = -(q1 + E[it.row + 1]) * is;
-                                const T l2 = -(q2 + E[it.row + 2]) * is;
-                                T lv[3];
-                                if (ln <= (T)0) {
-                                    lv[0] = lv[1] = lv[2] = (T)0;
-                                } else {
-                                    const T t2 = l1 * l1 + l2 * l2;
-                                    const T lim = MU[it.row] * ln;
-                                    lv[0] = ln;
-                                    if (t2 > lim * lim) { const T f = lim * rsq(t2); lv[1] = l1 * f; lv[2] = l2 * f; }
-                                    else { lv[1] = l1; lv[2] = l2; }
-                                }
-                                LAM[it.row] = lv[0]; LAM[it.row + 1] = lv[1]; LAM[it.row + 2] = lv[2];
-                                for (int s = 0; s < it.ns; ++s) {
-#pragma unroll
-                                    for (int r = 0; r < 3; ++r) {
-                                        const int t = ls[s] + r;
-                                        const T yv = Y[t], zo = Z[t];
-                                        const T zn = (yv + lv[r]) * INVB[t];
-                                        mloc = umax(mloc, umax(rbits(fabs(X[t] - zn)), rbits(fabs(zn - zo))));
-                                        ZO[t] = zo;
-                                        Z[t] = zn;
-                                        wn[t] = yv + (T)2 * lv[r];
-                                    }
-                                }
-                            } else {
-                                T q = (T)0;
-                                for (int s = 0; s < it.ns; ++s) q += Y[ls[s]] * INVB[ls[s]];
-                                const T e = E[it.row];
-                                T lv;
-                                if (it.type == TYPE_EQUALITY) lv = -(q + e) * INVS[it.row];
-                                else if (it.type == TYPE_HARD) { lv = -(q + e) * INVS[it.row]; lv = lv > (T)0 ? lv : (T)0; }
-                                else lv = -(e + AL[it.row] * q) * KF[it.row];
-                                LAM[it.row] = lv;
-                                for (int s = 0; s < it.ns; ++s) {
-                                    const int t = ls[s];
-                                    const T yv = Y[t], zo = Z[t];
-                                    const T zn = (yv + lv) * INVB[t];
-                                    mloc = umax(mloc, umax(rbits(fabs(X[t] - zn)), rbits(fabs(zn - zo))));
-                                    ZO[t] = zo;
-                                    Z[t] = zn;
-                                    wn[t] = yv + (T)2 * lv;
-                                }
-                            }
-                        }
-                    }
                     if (!(learned_mode && l == 9)) {
                         // the stop test rides on the barrier: the number of threads whose
                         // residual is finite and above the tolerance.  A non-finite iterate
@@ -2153,19 +2038,17 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                         if (primal_stop && over == 0) { conv = 1; break; }
                         continue;
                     }
-                    mloc = warp_umax(mloc);
-                    if (lane == 0) ured[l & 1][warp] = mloc;
+                    const U wmax = warp_umax(mloc);
+                    if (lane == 0) ured[warp] = wmax;
                     __syncthreads();
                     U mx = 0;
 #pragma unroll
-                    for (int q = 0; q < NW; ++q) mx = umax(mx, ured[l & 1][q]);
+                    for (int q = 0; q < NW; ++q) mx = umax(mx, ured[q]);
                     par ^= 1;
                     pc.mark(PHASE_ZSTEP);
-                    {
-                        if (learned && (unsigned long long)mx > ref10) { restart = true; break; }
-                        if (!learned && tid == 0) P.ref10[sc] = (unsigned long long)mx;
-                        if (learned && tid == 0) P.learn_skip[2 * sc + 1] = 0;   // kept: streak ends
-                    }
+                    if (learned && (unsigned long long)mx > ref10) { restart = true; break; }
+                    if (!learned && tid == 0) P.ref10[sc] = (unsigned long long)mx;
+                    if (learned && tid == 0) P.learn_skip[2 * sc + 1] = 0;       // kept: streak ends
                     if (mx >= inf_bits(T(0))) { status = ST_NAN; break; }
                     if (primal_stop && mx <= tolb) { conv = 1; break; }
                 }
@@ -2226,7 +2109,7 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                         tolc *= 0.5;
                         tolb = tol_bits(T(0), tolc);
                         if (CACHED && xv) { xc = V.htb[V.coff[xt]]; zreg = Z[xt]; }
-                            conv = 0;
+                        conv = 0;
                         ++l;
                         continue;
                     }
