@@ -62,7 +62,7 @@ struct LaunchClass {
 
 // A grid scene's layout for the iteration kernel (grid_iter.cuh), for one block count
 struct IterPlan {
-    int blocks = 0;                // the count it was built for (0: not built)
+    int blocks = 0;                // the count it was built for
     int nwaves = 0, per_block = 0; // nwaves 0: the scene has more side-rows than lanes
     bool wide = false;             // rows too wide for shared memory slots: the LONG kernel
     int row_share = 0;             // shared memory of a warp: its slots, or (LONG) the most bytes of
@@ -140,7 +140,9 @@ struct sim_s {
     std::vector<subadmm::CholPlan> chol;   // per scene: the blocked factorisation's panels
     std::vector<subadmm::BandPlan> band;   // per scene: the banded factorisation of its tc subsystems
     std::vector<int> h_ipool;      // host copy of the integer pool (envelopes)
-    std::vector<IterPlan> iter;            // per scene: grid scenes' iteration layout
+    // per scene: grid scenes' iteration layouts, one for every block count used so far (a graph that
+    // the caller captured keeps reading the one it was captured with)
+    std::vector<std::vector<IterPlan>> iter;
     std::vector<char> grid_tables;         // per scene: its tables are in the workspace
     std::vector<Item> h_items;             // host copies of the projection items
     std::vector<int> h_lists;
@@ -304,7 +306,8 @@ void free_device(sim_t s)
     for (auto &b : s->band) subadmm::band_plan_free(b);
     s->band.clear();
     s->grid_factored.clear();
-    for (auto &p : s->iter) { cudaFree(p.d_lane); cudaFree(p.d_head); cudaFree(p.d_tag); }
+    for (auto &v : s->iter)
+        for (auto &p : v) { cudaFree(p.d_lane); cudaFree(p.d_head); cudaFree(p.d_tag); }
     s->iter.clear();
     s->grid_tables.clear();
     if (s->graph_stream) cudaStreamDestroy(s->graph_stream);
@@ -338,7 +341,8 @@ int zeros(sim_t s, double **dst, size_t count, const char *what)
 }
 
 int iter_blocks(const sim_t s, int sms, int div);
-int iter_plan_of(sim_t s, int sc, int blocks);
+int iter_plan_of(sim_t s, int sc, int blocks, const IterPlan **out);
+int iter_plans(sim_t s);
 
 // Lays out every scene for the step kernel and uploads it.
 int finalize(sim_t s)
@@ -1076,7 +1080,7 @@ int finalize(sim_t s)
     s->h_ipool = ipool;
     s->h_items = items;
     s->h_lists = lists;
-    s->iter.assign(nscenes, IterPlan{});
+    s->iter.assign(nscenes, {});
     s->grid_tables.assign(nscenes, 0);
     {
         {
@@ -1110,13 +1114,7 @@ int finalize(sim_t s)
         if (e != cudaSuccess) return fail(s, SIM_ENOMEM, "cudaMalloc stats");
         CK(cudaMemsetAsync(s->d_stats, 0, std::max(1, 5 * nscenes) * sizeof(long long), s->stream), "memset stats");
     }
-    if (s->opt.stop != SIM_STOP_THETA) {
-        int sms = 0;
-        CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->opt.device), "attribute");
-        for (const LaunchClass &c : s->classes)
-            for (int sc : c.scenes)
-                if (c.grid && (rc = iter_plan_of(s, sc, iter_blocks(s, sms, c.block_div)))) return rc;
-    }
+    if ((rc = iter_plans(s))) return rc;
     s->finalized = true;
     return SIM_OK;
 }
@@ -1590,9 +1588,10 @@ int iter_blocks(const sim_t s, int sms, int div)
 // subsystems they join, cut into runs of nearly equal work (vectors of D, plus a constant per
 // row), whole items, at most 32 side-rows.  A wave is short when it has at most 8 rows of at
 // most 32 vectors (one per lane): as long as there are warps enough, runs are cut there.
-int iter_plan_of(sim_t s, int sc, int blocks)
+int iter_plan_of(sim_t s, int sc, int blocks, const IterPlan **out)
 {
-    if (s->iter[sc].blocks == blocks) return SIM_OK;
+    for (const IterPlan &p : s->iter[sc])
+        if (p.blocks == blocks) { *out = &p; return SIM_OK; }
     const SceneDesc &S = s->scenes[sc];
     const int vn = s->opt.precision == SIM_MIXED ? 4 : 2, warps = blocks * (SUBADMM_ITER / 32);
     std::vector<int> sub(S.nsr, 0);                  // subsystem of each side-row
@@ -1717,44 +1716,60 @@ int iter_plan_of(sim_t s, int sc, int blocks)
             head.push_back(H);
         }
     }
-    IterPlan &old = s->iter[sc];
-    if (old.d_lane) {
-        CK(cudaStreamSynchronize(s->stream), "iteration plan");     // launches that read the old one
-        cudaFree(old.d_lane);
-        cudaFree(old.d_head);
-        cudaFree(old.d_tag);
-        old = IterPlan{};
-    }
     if (P.nwaves > 0) {
-        if (cudaMalloc((void **)&P.d_lane, lane.size() * sizeof(WaveLane)) != cudaSuccess)
-            return fail(s, SIM_ENOMEM, "cudaMalloc iteration plan");
-        old = P;
-        if (cudaMalloc((void **)&P.d_head, head.size() * sizeof(WaveHead)) != cudaSuccess) {
-            old.blocks = 0;
-            return fail(s, SIM_ENOMEM, "cudaMalloc iteration plan");
-        }
-        CK(cudaMemcpy(P.d_lane, lane.data(), lane.size() * sizeof(WaveLane), cudaMemcpyHostToDevice), "iteration plan");
-        old = P;
-        CK(cudaMemcpy(P.d_head, head.data(), head.size() * sizeof(WaveHead), cudaMemcpyHostToDevice), "iteration plan");
+        // the tagged words of every side-row, twice: tag 0x80000000 matches no iteration, ~0
+        // marks padding side-rows (no owner, value 0)
+        std::vector<unsigned> tags;
         if (in_slots) {
             P.row_share = 512 * std::max(8, 3 * rv + 3);
-            // the tagged words of every side-row, twice: tag 0x80000000 matches no iteration, ~0
-            // marks padding side-rows (no owner, value 0)
             const int words = vn == 4 ? 2 : 4;
-            std::vector<unsigned> tags(4 + 2 * (size_t)S.nsr * words, 0u);
+            tags.assign(4 + 2 * (size_t)S.nsr * words, 0u);
             for (size_t t = 0; t < 2 * (size_t)S.nsr; ++t)
                 for (int k = 1; k < words; k += 2) tags[4 + t * words + k] = ~0u;
             for (const WaveLane &L : lane)
                 for (int half = 0; half < 2 && L.t >= 0; ++half)
                     for (int k = 1; k < words; k += 2)
                         tags[4 + ((size_t)half * S.nsr + L.t) * words + k] = 0x80000000u;
-            if (cudaMalloc((void **)&P.d_tag, tags.size() * 4) != cudaSuccess)
-                return fail(s, SIM_ENOMEM, "cudaMalloc iteration plan");
-            old = P;
-            CK(cudaMemcpy(P.d_tag, tags.data(), tags.size() * 4, cudaMemcpyHostToDevice), "iteration plan");
+        }
+        auto put = [](auto **dst, const auto &v) {
+            if (v.empty()) return cudaSuccess;
+            cudaError_t e = cudaMalloc((void **)dst, v.size() * sizeof(v[0]));
+            if (e == cudaSuccess) e = cudaMemcpy(*dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
+            return e;
+        };
+        cudaError_t e = put(&P.d_lane, lane);
+        if (e == cudaSuccess) e = put(&P.d_head, head);
+        if (e == cudaSuccess) e = put(&P.d_tag, tags);
+        if (e != cudaSuccess) {
+            cudaFree(P.d_lane);
+            cudaFree(P.d_head);
+            cudaFree(P.d_tag);
+            if (e == cudaErrorMemoryAllocation) return fail(s, SIM_ENOMEM, "cudaMalloc iteration plan");
+            CK(e, "iteration plan");
         }
     }
-    s->iter[sc] = P;
+    s->iter[sc].push_back(P);
+    *out = &s->iter[sc].back();
+    return SIM_OK;
+}
+
+// What the launches of the grid scenes need, before the first of them (which may be captured): their
+// iteration layouts for the current block count, and the plans of their refactorised blocks
+int iter_plans(sim_t s)
+{
+    if (s->opt.stop == SIM_STOP_THETA) return SIM_OK;
+    int sms = 0;
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->opt.device), "attribute");
+    for (const LaunchClass &c : s->classes)
+        for (int sc : c.scenes) {
+            if (!c.grid) break;
+            const IterPlan *plan = nullptr;
+            int rc = iter_plan_of(s, sc, iter_blocks(s, sms, c.block_div), &plan);
+            if (rc) return rc;
+            if (plan->nwaves == 0) continue;
+            if ((rc = gram_plan_of(s, sc)) || (rc = band_plan_of(s, sc))) return rc;
+            if (s->tc_factor && s->band[sc].njobs == 0 && s->gram[sc].njobs > 0 && (rc = chol_plan_of(s, sc))) return rc;
+        }
     return SIM_OK;
 }
 
@@ -1769,11 +1784,11 @@ int coop_launch(sim_t s, KernFn kf, int blocks, int threads, size_t dyn, StepPar
 }
 
 // The steps of one grid scene as setup and iteration launches (grid_iter.cuh).
-int launch_grid_fused(sim_t s, LaunchClass &c, StepParams P, cudaStream_t st, int sc, bool capturing)
+int launch_grid_fused(sim_t s, LaunchClass &c, StepParams P, cudaStream_t st, int sc, const IterPlan &plan,
+                      bool capturing)
 {
     const bool mixed = s->opt.precision == SIM_MIXED;
     const SceneDesc &S = s->scenes[sc];
-    const IterPlan &plan = s->iter[sc];
     const KernFn setup = mixed ? subadmm::grid_setup_f32() : subadmm::grid_setup_f64();
     const KernFn iter = mixed ? subadmm::grid_iter_f32(plan.wide) : subadmm::grid_iter_f64(plan.wide);
     // block solves of large subsystems: in the setup's shared memory if that leaves two blocks per
@@ -1865,11 +1880,12 @@ int launch_grid_class(sim_t s, LaunchClass &c, StepParams P, cudaStream_t st, in
     CK(cudaStreamIsCapturing(st, &capturing), "capture status");
     for (size_t i = 0; i < c.scenes.size(); ++i) {
         if (s->opt.stop != SIM_STOP_THETA) {
-            const int rc = iter_plan_of(s, c.scenes[i], iter_blocks(s, sms, c.block_div));
+            const IterPlan *plan = nullptr;
+            const int rc = iter_plan_of(s, c.scenes[i], iter_blocks(s, sms, c.block_div), &plan);
             if (rc) return rc;
-            if (s->iter[c.scenes[i]].nwaves > 0) {
+            if (plan->nwaves > 0) {
                 P.scene_ids = s->d_scene_ids + c.ids_off + (int)i;
-                const int rf = launch_grid_fused(s, c, P, st, c.scenes[i], capturing != cudaStreamCaptureStatusNone);
+                const int rf = launch_grid_fused(s, c, P, st, c.scenes[i], *plan, capturing != cudaStreamCaptureStatusNone);
                 if (rf) return rf;
                 continue;
             }
@@ -2425,7 +2441,12 @@ int sim_grid_blocks(sim_t s, int blocks)
     if (!s) return SIM_EINVAL;
     if (blocks < 0) return fail(s, SIM_EINVAL, "blocks must be >= 0");
     s->grid_blocks = blocks;
-    return SIM_OK;
+    if (!s->finalized) return SIM_OK;
+    // (the layouts for the new count now, so that the next step allocates nothing)
+    ON_DEVICE(s->opt.device);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(s->stream, &cs), "capture status");
+    return cs == cudaStreamCaptureStatusNone ? iter_plans(s) : SIM_OK;
 }
 
 int sim_set_solver(sim_t s, int solver, double omega)
