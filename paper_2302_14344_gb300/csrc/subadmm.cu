@@ -2173,14 +2173,27 @@ int sim_autotune(sim_t s, int steps, int max_classes, long long *out)
         bool bc = c.cached;
         int bs = c.split, bt = c.nt;
         if (c.grid) {
-            // lanes per side-row, and all resident blocks or half of them (unless the caller
-            // fixed the block count); half the blocks must win by 3% over all of them, as the
-            // short timing is noisy
+            // all resident blocks or half of them (unless the caller fixed the block count), and the
+            // lanes per side-row where a scene of the class takes the two-barrier launch, the only
+            // one that has them; half the blocks must win by 3% over all of them, as the short
+            // timing is noisy
             double best_div[3] = {1e300, 1e300, 1e300};
             int split_div[3] = {c.split, c.split, c.split};
+            const int given = c.split;
             for (int div = 1; div <= (s->grid_blocks > 0 ? 1 : 2) && err == cudaSuccess; ++div)
             for (int split = 8; split <= 32 && err == cudaSuccess; split *= 2) {
                 c.block_div = div;
+                bool lanes = s->opt.stop == SIM_STOP_THETA || given < 8;
+                for (size_t i = 0; i < c.scenes.size() && !lanes; ++i) {
+                    const IterPlan *plan = nullptr;
+                    int sms = 0;
+                    err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->opt.device);
+                    if (err == cudaSuccess && iter_plan_of(s, c.scenes[i], iter_blocks(s, sms, div), &plan))
+                        err = cudaErrorMemoryAllocation;
+                    if (err != cudaSuccess) break;
+                    lanes = plan->nwaves == 0;
+                }
+                if (err != cudaSuccess || (!lanes && split != given)) continue;
                 float ms = 0.0f;
                 for (int rep = 0; rep < 2 && err == cudaSuccess; ++rep) {   // warm, then timed
                     err = copy_all(false);
