@@ -32,8 +32,11 @@ struct wsn_s {
     std::vector<__nv_bfloat16 *> act;  // act[l]: input of layer l (B x sizes[l])
     std::vector<float *> pre;          // pre[l]: pre-activation of hidden layer l (B x sizes[l+1])
     float *y = nullptr;                // network output (B x out)
-    std::vector<__nv_bfloat16 *> gl;   // gl[l]: gradient of layer l's output (B x sizes[l+1])
-    float *part = nullptr;             // partial weight gradients of the batch's splits
+    __nv_bfloat16 *g0 = nullptr, *g1 = nullptr;   // layer gradients in turn (B x max width)
+    // from the first gradients on: gl[l], the gradient of layer l's output (B x sizes[l+1]; the last
+    // two layers' are g0 and g1), and the partial weight gradients of the batch's splits
+    std::vector<__nv_bfloat16 *> gl;
+    float *part = nullptr;
     int max_splits = 1;
     // fused tensor-core inference (the 32-256-256-256-7 warm-start shape): packed BF16
     // weights (K-major per layer), their tensor maps, the kernel's error word
@@ -63,16 +66,24 @@ int werr(wsn_t w, int code, const std::string &msg)
 
 int grid_for(long long n) { return (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 4096)); }
 
+void free_grads(wsn_t w)
+{
+    for (auto *q : w->gl)
+        if (q != w->g0 && q != w->g1) cudaFree(q);
+    w->gl.clear();
+    cudaFree(w->part);
+    w->part = nullptr;
+}
+
 void free_ws(wsn_t w)
 {
     for (auto *a : w->act) cudaFree(a);
     for (auto *q : w->pre) cudaFree(q);
     w->act.clear();
     w->pre.clear();
-    for (auto *q : w->gl) cudaFree(q);
-    w->gl.clear();
-    cudaFree(w->y); cudaFree(w->part);
-    w->y = nullptr; w->part = nullptr;
+    free_grads(w);
+    cudaFree(w->y); cudaFree(w->g0); cudaFree(w->g1);
+    w->y = nullptr; w->g0 = nullptr; w->g1 = nullptr;
     w->cap = 0;
 }
 
@@ -84,23 +95,46 @@ int reserve(wsn_t w, int batch)
     const int cap = std::max(batch, 1024);
     w->act.assign(L, nullptr);
     w->pre.assign(L, nullptr);
-    w->gl.assign(L, nullptr);
+    int wmax = 0;
+    for (int q : w->sizes) wmax = std::max(wmax, q);
+    for (int l = 0; l < L; ++l) {
+        WCK(cudaMalloc((void **)&w->act[l], sizeof(__nv_bfloat16) * (size_t)cap * w->sizes[l]), "cudaMalloc");
+        WCK(cudaMalloc((void **)&w->pre[l], sizeof(float) * (size_t)cap * w->sizes[l + 1]), "cudaMalloc");
+    }
+    WCK(cudaMalloc((void **)&w->y, sizeof(float) * (size_t)cap * w->sizes[L]), "cudaMalloc");
+    WCK(cudaMalloc((void **)&w->g0, sizeof(__nv_bfloat16) * (size_t)cap * wmax), "cudaMalloc");
+    WCK(cudaMalloc((void **)&w->g1, sizeof(__nv_bfloat16) * (size_t)cap * wmax), "cudaMalloc");
+    w->cap = cap;
+    w->ws_gen = ++g_ws_generation;
+    return SIM_OK;
+}
+
+// The buffers that let all layers' weight gradients go in one launch, split over the batch: a
+// network that is only evaluated does not hold them.  False where they cannot be had (a capture
+// allocates nothing; no memory): the layers then go one by one through g0 and g1.
+bool reserve_grads(wsn_t w, cudaStream_t st)
+{
+    if (w->part) return true;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
+    const int L = (int)w->sizes.size() - 1;
     // splits of the batch in the weight gradients: enough 64 x 64 tiles for two blocks per SM
     // and scheduling slot (about 600), at most 16 (each holds a whole partial gradient)
     long long tiles = 0;
     for (int l = 0; l < L; ++l)
         tiles += (long long)((w->sizes[l] + wsn::TM - 1) / wsn::TM) * ((w->sizes[l + 1] + wsn::TN - 1) / wsn::TN);
     w->max_splits = (int)std::max<long long>(1, std::min<long long>(16, (600 + tiles - 1) / tiles));
-    WCK(cudaMalloc((void **)&w->part, sizeof(float) * (size_t)w->nparams * w->max_splits), "cudaMalloc");
+    w->gl.assign(L, nullptr);
+    bool ok = cudaMalloc((void **)&w->part, sizeof(float) * (size_t)w->nparams * w->max_splits) == cudaSuccess;
     for (int l = 0; l < L; ++l) {
-        WCK(cudaMalloc((void **)&w->act[l], sizeof(__nv_bfloat16) * (size_t)cap * w->sizes[l]), "cudaMalloc");
-        WCK(cudaMalloc((void **)&w->pre[l], sizeof(float) * (size_t)cap * w->sizes[l + 1]), "cudaMalloc");
-        WCK(cudaMalloc((void **)&w->gl[l], sizeof(__nv_bfloat16) * (size_t)cap * w->sizes[l + 1]), "cudaMalloc");
+        if (l >= L - 2) w->gl[l] = l == L - 1 ? w->g0 : w->g1;
+        else ok = ok && cudaMalloc((void **)&w->gl[l], sizeof(__nv_bfloat16) * (size_t)w->cap * w->sizes[l + 1]) == cudaSuccess;
     }
-    WCK(cudaMalloc((void **)&w->y, sizeof(float) * (size_t)cap * w->sizes[L]), "cudaMalloc");
-    w->cap = cap;
-    w->ws_gen = ++g_ws_generation;
-    return SIM_OK;
+    if (!ok) {
+        cudaGetLastError();
+        free_grads(w);
+    }
+    return ok;
 }
 
 // operands of a product, and whether their rows can be copied 16 bytes at a time
@@ -154,39 +188,48 @@ int backward(wsn_t w, const float *t, const float *mask, int batch, float *grad,
 {
     const int L = (int)w->sizes.size() - 1;
     const int N = w->sizes[L];
+    const bool whole = reserve_grads(w, st);
+    auto gl = [&](int l) { return whole ? w->gl[l] : (L - 1 - l) % 2 ? w->g1 : w->g0; };
     wsn::output_grad_kernel<<<grid_for((long long)batch * N), 256, 0, st>>>(
-        w->y, t, mask, w->scale, w->gl[L - 1], batch, N, loss);
+        w->y, t, mask, w->scale, gl(L - 1), batch, N, loss);
     WCK(cudaGetLastError(), "output grad launch");
     int rc;
-    for (int l = L - 1; l > 0; --l) {           // g_prev = (g W^T) * GELU'(pre)
-        const int in = w->sizes[l], out = w->sizes[l + 1];
-        wsn::Gemm ga = operands(w->gl[l], out, w->pb + w->w_off[l], out);
-        ga.M = batch; ga.N = in; ga.K = out;
-        ga.pre = w->pre[l - 1];
-        ga.act = w->gl[l - 1];
-        if ((rc = gemm<wsn::EPI_GELU_BWD, true>(w, ga, st))) return rc;
-    }
-    // dW = act^T g and db = column sums of g, the batch in splits of at least 128 rows
-    int chunk = (batch + w->max_splits - 1) / w->max_splits;
+    // dW = act^T g and db = column sums of g of `layers` layers, the batch in splits of at least 128 rows
+    const int most = whole ? w->max_splits : 1;
+    int chunk = (batch + most - 1) / most;
     chunk = std::max(128, (chunk + wsn::TK - 1) / wsn::TK * wsn::TK);
     const int splits = (batch + chunk - 1) / chunk;
-    for (int l0 = 0; l0 < L; l0 += wsn::kGroup) {
+    auto wgrad = [&](int l0, int layers) -> int {
         wsn::WgradGroup q{};
-        q.layers = std::min(L - l0, wsn::kGroup);
+        q.layers = layers;
         q.chunk = chunk;
         q.stride = w->nparams;
         q.part = splits == 1 ? grad : w->part;
-        for (int k = 0; k < q.layers; ++k) {
+        for (int k = 0; k < layers; ++k) {
             const int l = l0 + k, in = w->sizes[l], out = w->sizes[l + 1];
-            q.g[k] = operands(w->act[l], in, w->gl[l], out);
+            q.g[k] = operands(w->act[l], in, gl(l), out);
             q.g[k].M = in; q.g[k].N = out; q.g[k].K = batch;
             q.woff[k] = w->w_off[l];
             q.boff[k] = w->b_off[l];
             q.tile0[k + 1] = q.tile0[k] + (in + wsn::TM - 1) / wsn::TM * ((out + wsn::TN - 1) / wsn::TN);
         }
-        wsn::wgrad_kernel<<<dim3(q.tile0[q.layers], splits), 128, 0, st>>>(q);
+        wsn::wgrad_kernel<<<dim3(q.tile0[layers], splits), 128, 0, st>>>(q);
         WCK(cudaGetLastError(), "weight gradient launch");
+        return SIM_OK;
+    };
+    for (int l = L - 1; l >= 0; --l) {
+        if (!whole && (rc = wgrad(l, 1))) return rc;
+        if (l == 0) break;
+        const int in = w->sizes[l], out = w->sizes[l + 1];          // g_prev = (g W^T) * GELU'(pre)
+        wsn::Gemm ga = operands(gl(l), out, w->pb + w->w_off[l], out);
+        ga.M = batch; ga.N = in; ga.K = out;
+        ga.pre = w->pre[l - 1];
+        ga.act = gl(l - 1);
+        if ((rc = gemm<wsn::EPI_GELU_BWD, true>(w, ga, st))) return rc;
     }
+    if (!whole) return SIM_OK;
+    for (int l0 = 0; l0 < L; l0 += wsn::kGroup)
+        if ((rc = wgrad(l0, std::min(L - l0, wsn::kGroup)))) return rc;
     if (splits > 1) {
         wsn::grad_reduce_kernel<<<grid_for(w->nparams), 256, 0, st>>>(w->part, w->nparams, splits, grad,
                                                                        w->nparams);
