@@ -97,6 +97,115 @@ __device__ __forceinline__ void drain_stages(unsigned long long *bars, unsigned 
     }
 }
 
+// One z-step item held in a thread's registers for a whole step (items with at most two
+// sides): its type, row, side-rows and the step's constants (z is read and written in memory
+// each iteration).
+template <typename T>
+struct RegItem {
+    using U = typename VecOf<T>::U;
+    bool valid = false;
+    int type = 0, row = 0, t0 = 0, t1 = -1, nr = 1;
+    T ib0 = (T)0, ib1 = (T)0, e0 = (T)0, e1 = (T)0, e2 = (T)0;
+    T is = (T)0, kf = (T)0, al = (T)0, mu = (T)0;
+
+    __device__ __forceinline__ void load(const Item *items, const int *list, int i, const T *INVB,
+                                         const T *E, const T *INVS, const T *KF, const T *AL,
+                                         const T *MU)
+    {
+        const Item it = items[i];
+        if (it.type < 0) return;
+        valid = true;
+        type = it.type;
+        row = it.row;
+        t0 = list[it.lo];
+        t1 = it.ns > 1 ? list[it.lo + 1] : -1;
+        nr = type == TYPE_CONTACT ? 3 : 1;
+        ib0 = INVB[t0];
+        if (t1 >= 0) ib1 = INVB[t1];
+        e0 = E[row];
+        if (nr == 3) { e1 = E[row + 1]; e2 = E[row + 2]; }
+        is = INVS[row]; kf = KF[row]; al = AL[row]; mu = MU[row];
+    }
+
+    // z of side-row t, replaced by zn; returns the old z
+    static __device__ __forceinline__ T swap_z(T *Z, T *ZO, int t, T zn)
+    {
+        const T zo = Z[t];
+        ZO[t] = zo;
+        Z[t] = zn;
+        return zo;
+    }
+
+    // the item's projection (Sec. III-C): lambda, z, w of the next v-step; returns the bits
+    // of max(|x - z|, |dz|) over its side-rows
+    __device__ __forceinline__ U project(const T *Y, const T *X, T *LAM, T *wn, T *Z, T *ZO)
+    {
+        U mloc = 0;
+        if (!valid) return mloc;
+        if (type == TYPE_CONTACT) {
+            T ya[3], yb[3] = {(T)0, (T)0, (T)0};
+#pragma unroll
+            for (int r = 0; r < 3; ++r) ya[r] = Y[t0 + r];
+            if (t1 >= 0) {
+#pragma unroll
+                for (int r = 0; r < 3; ++r) yb[r] = Y[t1 + r];
+            }
+            const T ln = -(ya[0] * ib0 + yb[0] * ib1 + e0) * is;
+            const T l1 = -(ya[1] * ib0 + yb[1] * ib1 + e1) * is;
+            const T l2 = -(ya[2] * ib0 + yb[2] * ib1 + e2) * is;
+            T lv[3];
+            if (ln <= (T)0) {
+                lv[0] = lv[1] = lv[2] = (T)0;
+            } else {
+                const T t2 = l1 * l1 + l2 * l2;
+                const T lim = mu * ln;
+                lv[0] = ln;
+                if (t2 > lim * lim) { const T f = lim * rsq(t2); lv[1] = l1 * f; lv[2] = l2 * f; }
+                else { lv[1] = l1; lv[2] = l2; }
+            }
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                LAM[row + r] = lv[r];
+                const T zn = (ya[r] + lv[r]) * ib0;
+                const T zo = swap_z(Z, ZO, t0 + r, zn);
+                mloc = umax(mloc, umax(rbits(fabs(X[t0 + r] - zn)), rbits(fabs(zn - zo))));
+                wn[t0 + r] = ya[r] + (T)2 * lv[r];
+            }
+            if (t1 >= 0) {
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    const T zn = (yb[r] + lv[r]) * ib1;
+                    const T zo = swap_z(Z, ZO, t1 + r, zn);
+                    mloc = umax(mloc, umax(rbits(fabs(X[t1 + r] - zn)), rbits(fabs(zn - zo))));
+                    wn[t1 + r] = yb[r] + (T)2 * lv[r];
+                }
+            }
+        } else {
+            const T y0 = Y[t0];
+            const T y1 = t1 >= 0 ? Y[t1] : (T)0;
+            const T q = y0 * ib0 + y1 * ib1;
+            T lv;
+            if (type == TYPE_SOFT) lv = -(e0 + al * q) * kf;
+            else {
+                lv = -(q + e0) * is;
+                if (type == TYPE_HARD) lv = lv > (T)0 ? lv : (T)0;
+            }
+            LAM[row] = lv;
+            const T zn0 = (y0 + lv) * ib0;
+            const T zo0 = swap_z(Z, ZO, t0, zn0);
+            mloc = umax(mloc, umax(rbits(fabs(X[t0] - zn0)), rbits(fabs(zn0 - zo0))));
+            wn[t0] = y0 + (T)2 * lv;
+            if (t1 >= 0) {
+                const T zn1 = (y1 + lv) * ib1;
+                const T zo1 = swap_z(Z, ZO, t1, zn1);
+                mloc = umax(mloc, umax(rbits(fabs(X[t1] - zn1)), rbits(fabs(zn1 - zo1))));
+                wn[t1] = y1 + (T)2 * lv;
+            }
+        }
+        return mloc;
+    }
+};
+
 template <typename T, int SPLIT>
 __global__ void __launch_bounds__(SUBADMM_THREADS, 2) grid_step_kernel(StepParams P)
 {
@@ -188,11 +297,11 @@ __global__ void __launch_bounds__(SUBADMM_THREADS, 2) grid_step_kernel(StepParam
         // items spreads them over the SMs rather than filling the first blocks.
         const int ix = 32 * d.warp + lane;
         const bool icache = S.nitem <= d.nthreads && !P.pj;
-        RegItem<T, false> ri;
+        RegItem<T> ri;
         bool igeneric = false;
         if (icache && ix < S.nitem) {
             const Item it = V.item[ix];
-            if (it.ns <= 2) ri.load(V.item, V.list, ix, INVB, E, INVS, KF, AL, MU, Z);
+            if (it.ns <= 2) ri.load(V.item, V.list, ix, INVB, E, INVS, KF, AL, MU);
             else igeneric = it.type >= 0;
         }
         // initial z, u = -lambda; a learned start is checked after 10 iterations against the
