@@ -193,9 +193,9 @@ int sim_step(sim_t s, int n_steps);
  * grid, 3 generic with 512 threads per block: a class whose scenes take a whole SM's shared
  * memory, so that a block has the whole register file and twice the warps), lanes per
  * side-row (1, 2 or 4; for the grid kernels 8, 16 or 32, which the launch of all steps with two
- * barriers an iteration uses), dynamic shared memory per block in bytes (for a grid class: the shared memory for its D rows at its last
- * launch, 0 before the first, without staging, or if all its rows are short; see
- * sim_grid_staging), 0.  Returns the number
+ * barriers an iteration uses), dynamic shared memory per block in bytes (for a grid class: the
+ * shared memory for its D rows at its last launch; 0 before the first and, where rows are long,
+ * without staging; see sim_grid_staging), 0.  Returns the number
  * of classes, or a negative SIM_E* code.
  * sim_autotune times, for each class on its own, every kernel variant that is valid for all
  * its scenes (generic with 1, 2 or 4 lanes per side-row and 256 or 512 threads per block,
@@ -260,7 +260,7 @@ int sim_grid_threshold(sim_t s, int side_rows);
 /* Grid kernels: with enable != 0 (the default) each warp of the iteration launch keeps as many
  * of its long D rows in shared memory for the step as fit its share, and streams the others
  * (the two-barrier launch: every D row staged by bulk asynchronous copies, two stages per
- * warp); with 0 the rows are read from global memory directly.  The results are the same
+ * warp); with 0 those rows are read from global memory directly.  The results are the same
  * either way (the same products in the same order).  Takes effect at the next sim_step. */
 int sim_grid_staging(sim_t s, int enable);
 

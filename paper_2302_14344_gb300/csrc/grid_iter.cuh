@@ -333,14 +333,17 @@ __global__ void __launch_bounds__(SUBADMM_ITER, 1) grid_iter_kernel(const __grid
     constexpr bool MIXED = sizeof(T) == 4;
     // vectors of a row per lane and segment (LONG): a row ahead of FP32 for the latency of its
     // stream (3 in place of 6: 17.9 -> 21.5 us an iteration of 64 slabs); in FP64 the three buffers
-    // of 6 did not fit the registers, and 3 still cover the pipe (72k -> 47k cycles, 16 slabs)
+    // of 6 did not fit the registers, and 3 still cover the pipe (v-step of 16 slabs 72k -> 47k cycles,
+    // the iteration 77k -> 51k)
     constexpr int CH = MIXED ? 6 : 3;
     constexpr int RV = kWideVecs<T>();             // vectors per lane of a wide row (shape B)
     static_assert(RV <= 4, "a wide row's w is gathered at once");
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(128) unsigned char smem[];
-    // (what the loop does not use lives in shared memory: its registers must not spill, as 512
-    // threads' frames do not fit L1 next to the D rows)
+    // (what the loop does not use lives in shared memory, to spill less: 512 threads' frames do not
+    // fit L1 next to the D rows.  What is left, by -Xptxas -v: some 580 bytes of spill stores a
+    // thread in FP32 without LONG, 440 with, 190 and 110 in FP64; with 860-byte frames in the
+    // loop a stir iteration took 13k cycles, now 8.4k)
     __shared__ SceneDesc S;
     __shared__ View<T> V;
     __shared__ IterBarrier bar;
@@ -662,7 +665,7 @@ __global__ void __launch_bounds__(SUBADMM_ITER, 1) grid_iter_kernel(const __grid
             const T dl = la - lam;
             U mloc = 0;
             // (a learned start's check after 10 iterations needs the z of the ninth, too)
-            if (primal_stop || (learned_mode && (l == 8 || l == 9))) {
+            if (primal_stop || (learned_mode && (unsigned)(l - 8) < 2u)) {
                 const T zn = xn + dl * ib;
                 if (own) mloc = umax(rbits(fabs(dl * ib)), rbits(fabs(zn - z)));
                 z = zn;
@@ -700,8 +703,10 @@ __global__ void __launch_bounds__(SUBADMM_ITER, 1) grid_iter_kernel(const __grid
                 }
                 over = bar.sync(over);
                 pc.mark(trace, PHASE_ZSTEP);
-                if (over >> 16) { status = ST_NAN; break; }
-                if (primal_stop && over == 0) { conv = 1; break; }
+                if (primal_stop) {
+                    if (over >> 16) { status = ST_NAN; break; }
+                    if (over == 0) { conv = 1; break; }
+                }
                 continue;
             }
             mloc = warp_umax(mloc);

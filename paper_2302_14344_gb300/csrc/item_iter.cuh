@@ -4,7 +4,9 @@
 // v-step (lane groups, two side-rows per trip: independent load and FMA chains overlap), a barrier,
 // z-step (a thread per projection item, the item's y, x and z through shared memory), a barrier.
 // A call of its own, like own_iterate: inline, its tables and the code around it spilled each
-// other's registers (step_kernel<double>: 280 bytes of spill stores around the calls).
+// other's registers (280 bytes of spill stores in FP64; here none).  Explicit blocks of 3 sides,
+// FP64: 8.9k -> 7.7k cycles an iteration.  Plain arguments, no struct by value: nvcc 13.0 handed a
+// struct of ints, bools and two T on with other fields' values.
 #pragma once
 #include "layout.h"
 

@@ -8,10 +8,10 @@
 // grid_iter.cuh).  The item loop that this replaces gathered and scattered y, z, lambda and the
 // tables of every item in every iteration, 16 FP64 instructions a row where 6 do.
 //
-// A call of its own: the step kernel around it holds 1.4 KB of frames per thread, and with the
+// A call of its own: the step kernel around it holds 0.8 KB of frames per thread, and with the
 // shared memory full the L1 is too small for any spill inside the loop (the loop inline spilled
 // its rows' state and took 7.2k cycles an iteration on the batched scenes, the item loop 7.6k; this
-// takes 4.5k).  Offsets from the block's shared memory, not pointers, so that its accesses are
+// takes 4.4k).  Offsets from the block's shared memory, not pointers, so that its accesses are
 // shared-memory instructions.
 #pragma once
 #include "layout.h"

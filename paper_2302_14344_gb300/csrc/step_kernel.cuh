@@ -31,8 +31,8 @@
 // difference of x at the current iterate (iterative refinement) and the iterations resume.
 //
 // On GB300 an FP64 warp instruction costs about 64 issue cycles of a sub-partition however
-// few lanes are active, so FP64 work is kept out of the loop of the mixed form and the loop
-// keeps each thread's coefficients, y and z in registers for the whole step.
+// few lanes are active, so FP64 work is kept out of the loop of the mixed form and the loops
+// keep each thread's coefficients and lambda in registers for the whole step.
 #pragma once
 #include "layout.h"
 #include "rigid_model.cuh"
@@ -1665,10 +1665,10 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
             // ---- per-thread state of the register-cached iteration (CACHED).  The host's
             // thread map gives each thread a side-row (its lane group of SPLIT lanes) and puts
             // every projection item's side-rows on adjacent groups of one warp.  A thread keeps
-            // its side-row's D chunks, c, beta, 1/beta, x, y, z and lambda in registers and the
-            // constants of its item: the warp forms the items' y, and every lane of an item
-            // projects it (Sec. III-C) from y gathered by shuffles, so an iteration needs one
-            // block barrier (the new w) instead of two.
+            // its side-row's D chunks, c, beta, 1/beta, x and the lambda of the last iterations in
+            // registers, and the constants of its item: the warp forms x, every lane of an item
+            // gets its partner's x (a contact: its rows' lambda) by shuffles and projects its own row
+            // (Sec. III-C), so an iteration needs one block barrier (the new w) instead of two.
             // The updates are those of grid_iter.cuh: with d = lambda' - lambda, neither y nor z is
             // formed in the loop (z only for the stop test): 2 x chunks + 6 FP64 instructions per
             // warp and iteration (+ 1 while the stop test fails), each of which holds the FP64 pipe for 64
