@@ -1789,7 +1789,14 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                     const T l0 = __shfl_sync(0xffffffffu, la, fbase);
                     const T l1 = __shfl_sync(0xffffffffu, la, (fbase + SPLIT) & 31);
                     const T l2 = __shfl_sync(0xffffffffu, la, (fbase + 2 * SPLIT) & 31);
-                    if (ftype == TYPE_CONTACT) {
+                    if (sizeof(T) == 4) {
+                        // (no branches: they cost the warp that holds a sliding foot, which the block
+                        // waits for, some 140 cycles an iteration; FP64 instructions cost more)
+                        const T t2 = l1 * l1 + l2 * l2, lim = fmu * l0;
+                        const T f = above0(t2 - lim * lim) ? lim * rsq(t2) : (T)1;
+                        const T lc = !above0(l0) ? (T)0 : fr == 0 ? la : la * f;
+                        la = ftype == TYPE_CONTACT ? lc : la;
+                    } else if (ftype == TYPE_CONTACT) {
                         if (!above0(l0)) {
                             la = (T)0;
                         } else if (fr > 0) {
@@ -1810,7 +1817,7 @@ __global__ void __launch_bounds__(NT, (CACHED || NT > SUBADMM_THREADS) ? 1 : 2) 
                         over = xv && (unsigned long long)rbits(fabs(dl)) - blo < bspan;
                         if (over) res = btol_over;
                     }
-                    if (!__any_sync(0xffffffffu, over)) {
+                    if (sizeof(T) == 4 || !__any_sync(0xffffffffu, over)) {
                         const T dz = dl * xib, zn = acc + dz;
                         const T zo = !first ? xx + (lreg - lreg1) * xib : zreg;
                         if (xv && xgl == 0) res = umax(rbits(fabs(dz)), rbits(fabs(zn - zo)));
