@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(SUBADMM_ITER, 1) grid_iter_kernel(const __grid
             const T dl = la - lam;
             U mloc = 0;
             // (a learned start's check after 10 iterations needs the z of the ninth, too)
-            if (primal_stop || (learned_mode && (unsigned)(l - 8) < 2u)) {
+            if (primal_stop || (learned_mode && l <= 9)) {
                 const T zn = xn + dl * ib;
                 if (own) mloc = umax(rbits(fabs(dl * ib)), rbits(fabs(zn - z)));
                 z = zn;
